@@ -176,7 +176,7 @@ struct lbpc_handle {
         void* tape_m = nullptr;
         void* lam[2] = {nullptr, nullptr};
         double *gtw = nullptr, *Lpart = nullptr, *Jpart = nullptr, *red = nullptr;
-        int nblocks = 0;
+        int nblocks = 0, nwarps = 0;
     } adj;
     Args args;
     std::string err;
@@ -650,7 +650,7 @@ namespace {
 struct AdjLayout {
     size_t ckpt_bytes, off_f, off_g, off_hp, ckpt, tape_e, tape_m, lam0, lam1, gtw, Lpart, Jpart,
         red, total;
-    int nseg, nblocks;
+    int nseg, nblocks, nwarps;
 };
 
 AdjLayout adj_layout(const lbpc_handle* h, int nsteps, int k) {
@@ -675,7 +675,8 @@ AdjLayout adj_layout(const lbpc_handle* h, int nsteps, int k) {
     for (int f = 0; f < 6; f++) amax = std::max(amax, (size_t)face_area(h->nx, h->ny, h->nz, f));
     L.gtw = off; off = align_up(off + 8 * amax);
     L.nblocks = node_grid_blocks(h->nx, h->ny, h->nz);
-    L.Lpart = off; off = align_up(off + 8 * (size_t)L.nblocks * ADJ_WARPS_PER_BLOCK);
+    L.nwarps = node_grid_warps(h->nx, h->ny, h->nz);
+    L.Lpart = off; off = align_up(off + 8 * (size_t)L.nwarps);
     L.Jpart = off; off = align_up(off + 8 * (size_t)L.nblocks);
     L.red = off; off = align_up(off + 8 * 4);
     L.total = off;
@@ -722,6 +723,7 @@ lbpc_status lbpc_adjoint_forward(lbpc_handle* h, int nsteps, int ckpt_every, voi
     A.k = ckpt_every;
     A.nseg = L.nseg;
     A.nblocks = L.nblocks;
+    A.nwarps = L.nwarps;
     A.ckpt_bytes = L.ckpt_bytes;
     A.off_f = L.off_f; A.off_g = L.off_g; A.off_hp = L.off_hp;
     A.ckpt = w + L.ckpt;
@@ -828,7 +830,7 @@ lbpc_status lbpc_adjoint_backward(lbpc_handle* h, int face, double* dJ_dTw_host,
         }
         h->launches += len;
     }
-    k_sum<<<1, 256, 0, h->stream>>>(A.Lpart, A.nblocks * ADJ_WARPS_PER_BLOCK, A.red + 1);
+    k_sum<<<1, 256, 0, h->stream>>>(A.Lpart, A.nwarps, A.red + 1);
     h->launches++;
     LBPC_CK(h, cudaGetLastError());
     double dJdL = 0.0;

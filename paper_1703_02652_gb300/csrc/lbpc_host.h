@@ -212,6 +212,11 @@ inline void fill_args(Args& a, int nx, int ny, int nz, const lbpc_params& p, con
                       double* const Tw[6]) {
     std::memset(&a, 0, sizeof a);
     a.nx = nx; a.ny = ny; a.nz = nz; a.N = nx * ny * nz;
+    a.by_nx = fast_div(nx);
+    a.by_hx = fast_div(nx > 1 ? nx / 2 : 1);
+    a.by_ny = fast_div(ny);
+    a.fill_nx = rows_fill(nx, ny);
+    a.fill_hx = nx > 1 && rows_fill(nx / 2, ny);
     for (int ax = 0; ax < 3; ax++) a.per[ax] = p.bc[2 * ax] == LBPC_PERIODIC;
     for (int f = 0; f < 6; f++) {
         a.wall[f] = p.bc[f] != LBPC_PERIODIC;

@@ -41,8 +41,33 @@ struct Coef {
     C j_k_e, j_k_eps, j_k_q, j_k_nu9, j_k_pi10, j_k_nu11, j_k_pi12, j_k_nu13, j_k_t;
 };
 
+constexpr int STEP_THREADS = 128;  // threads of a block of the per-node and pair kernels
+
+// Division of n < 2^31 by a fixed d >= 1 through one high product (round-up reciprocal:
+// m = ceil(2^(31 + l) / d), l = ceil(log2 d), so that m d - 2^(31 + l) < d <= 2^l).
+struct FastDiv {
+    unsigned m, l;
+    __host__ __device__ unsigned div(unsigned n) const {
+#if defined(__CUDA_ARCH__)
+        return __umulhi(n << 1, m) >> l;
+#else
+        return (unsigned)((((unsigned long long)(n << 1) * m) >> 32) >> l);
+#endif
+    }
+};
+inline FastDiv fast_div(int d) {
+    FastDiv f{0, 0};
+    while ((1ull << f.l) < (unsigned long long)d) f.l++;
+    f.m = (unsigned)(((1ull << (31 + f.l)) + d - 1) / d);
+    return f;
+}
+
 struct Args {
     int nx, ny, nz, N;   // N = nx*ny*nz < 2^31
+    // item indices to (column, y, z), hx = nx / 2, and whether rows of nodes or pairs fill
+    // whole blocks
+    FastDiv by_nx, by_hx, by_ny;
+    int fill_nx, fill_hx;
     int per[3];          // periodic axes
     int wall_iso[6];     // face is an isothermal wall (anti-bounce-back of g)
     int wall[6];         // face is a wall (not periodic)
@@ -101,17 +126,38 @@ struct Launchers {
     size_t compute_bytes;  // bytes of one compute-precision value (adjoint, tape)
 };
 
-// node grid of the per-node kernels (blocks of 128 threads along x, then y)
-inline dim3 node_block_dims(int nx) {
-    const int bx = nx >= 128 ? 128 : (nx > 32 ? 64 : 32);
-    return dim3(bx, 128 / bx, 1);
+// Launch shape of the kernels that give each node (cols = nx) or node pair (cols = nx / 2)
+// a thread, in blocks of STEP_THREADS: whole rows where they fill blocks, otherwise items
+// counted in memory order (see item_cyz).  With planes of less
+// than eight blocks the count runs through the whole lattice (a second division per thread)
+// instead of starting anew at each z.  (Blocks of 32 or 64 on small lattices measured the
+// same: the step's latency does not depend on them.)
+constexpr int SM_COUNT = 152;
+// rows_fill: rows of cols items (with ny of them in a plane) fill whole blocks.
+struct ItemGrid { dim3 grid, block; };
+inline int block_rows(int cols) { return cols < STEP_THREADS ? STEP_THREADS / cols : 1; }
+inline bool rows_fill(int cols, int ny) {
+    if (cols % STEP_THREADS != 0 && (STEP_THREADS % cols != 0 || cols < 8)) return false;
+    return ny % block_rows(cols) == 0 || ny >= 8 * block_rows(cols);
 }
-// The adjoint's dJ/dL partials: one slot per warp of every block of the per-node grid
-// (blocks of 128 threads), so the reverse sweep reduces within warps only.
-constexpr int ADJ_WARPS_PER_BLOCK = 4;
+inline ItemGrid item_grid(int cols, int ny, int nz) {
+    const long long plane = (long long)cols * ny, all = plane * nz;
+    constexpr int t = STEP_THREADS;
+    if (rows_fill(cols, ny)) {
+        const int by = block_rows(cols), bx = t / by;
+        return {dim3(cols / bx, (ny + by - 1) / by, nz), dim3(bx, by)};
+    }
+    if (plane < 8 * t || nz == 1) return {dim3((unsigned)((all + t - 1) / t)), dim3(t)};
+    return {dim3((unsigned)((plane + t - 1) / t), nz), dim3(t)};
+}
+// Blocks and warps of the per-node grid: the adjoint keeps one partial of J per block and one
+// of dJ/dL per warp, so that the reverse sweep reduces within warps only.
 inline int node_grid_blocks(int nx, int ny, int nz) {
-    const dim3 b = node_block_dims(nx);
-    return ((nx + b.x - 1) / b.x) * ((ny + b.y - 1) / b.y) * nz;
+    const ItemGrid g = item_grid(nx, ny, nz);
+    return (int)(g.grid.x * g.grid.y * g.grid.z);
+}
+inline int node_grid_warps(int nx, int ny, int nz) {
+    return node_grid_blocks(nx, ny, nz) * (STEP_THREADS / 32);
 }
 
 const Launchers& launchers_f64();

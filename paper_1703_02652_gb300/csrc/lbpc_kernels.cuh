@@ -247,11 +247,23 @@ LBPC_HD C abb_source(const Args& a, const Coef<C>& k, int face, int x, int y, in
     return k.wT_cref * (C)a.Tw[face][face_index(a, face, x, y, z)] - C(2) * k.gshift;
 }
 
+// Anti-bounce-back of the outgoing value v (see abb_source).  FP64, never shifted: one fused
+// operation on the FP64 pipe instead of three.
+template <class C>
+LBPC_HD C abb_back(const Args& a, const Coef<C>& k, int face, int x, int y, int z, C v) {
+    if constexpr (sizeof(C) == 8)
+        return std::fma(k.wT_cref, a.Tw[face][face_index(a, face, x, y, z)], -v);
+    else
+        return -v + abb_source(a, k, face, x, y, z);
+}
+
 // ---------------------------------------------------------------------------------
 // Gathers: pre-collision populations of node n for each memory layout.
 // ---------------------------------------------------------------------------------
-// 16-bit populations (and pairs of them): read-only loads that ask L2 to fetch 256 bytes
-// around each miss; other types: plain read-only loads.
+// Loads of the pull gathers.  16-bit populations (and pairs of them) ask L2 to fetch 256
+// bytes around each miss.  They are plain loads, not read-only (.nc) ones: a step's blocks
+// become resident while the step before still writes what they will read, so the data is
+// not constant over the kernel's lifetime (both kinds measured the same, 64^3 to 256^3).
 template <class X> struct Is16 { static constexpr bool value = false; };
 template <> struct Is16<__half> { static constexpr bool value = true; };
 template <> struct Is16<__nv_bfloat16> { static constexpr bool value = true; };
@@ -259,38 +271,38 @@ template <> struct Is16<__half2> { static constexpr bool value = true; };
 template <> struct Is16<__nv_bfloat162> { static constexpr bool value = true; };
 #if defined(__CUDA_ARCH__)
 template <class X>
-__device__ __forceinline__ X ld_nc(const X* p) {
+__device__ __forceinline__ X ld_hint(const X* p) {
     if constexpr (Is16<X>::value && sizeof(X) == 2) {
         unsigned short v;
-        asm("ld.global.nc.L2::256B.u16 %0, [%1];" : "=h"(v) : "l"(p));
+        asm volatile("ld.global.L2::256B.u16 %0, [%1];" : "=h"(v) : "l"(p));
         return *reinterpret_cast<X*>(&v);
     } else if constexpr (Is16<X>::value && sizeof(X) == 4) {
         unsigned v;
-        asm("ld.global.nc.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
+        asm volatile("ld.global.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
         return *reinterpret_cast<X*>(&v);
     } else {
-        return __ldg(p);
+        return *p;
     }
 }
 #endif
-template <int P, int LAYOUT, bool NC>
+template <int P, int LAYOUT, bool HINT>
 LBPC_HD typename Store<P>::T ldv(const typename Store<P>::T* p) {
 #if defined(__CUDA_ARCH__)
-    if constexpr (NC) return ld_nc(p);
+    if constexpr (HINT) return ld_hint(p);
 #endif
     return *p;
 }
 
-// Load of any type through the read-only path (device, NC) or plainly.
-template <bool NC, class X>
+// Load of any type, with the 16-bit hint (device) or without.
+template <bool HINT, class X>
 LBPC_HD X ld_any(const X* p) {
 #if defined(__CUDA_ARCH__)
-    if constexpr (NC) return ld_nc(p);
+    if constexpr (HINT) return ld_hint(p);
 #endif
     return *p;
 }
 
-template <int P, int LAYOUT, bool NC, class NB>
+template <int P, int LAYOUT, bool HINT, class NB>
 LBPC_HD void gather_f(const Args& a, const NB& b, int n,
                                          const typename Store<P>::T* fs,
                                          typename Store<P>::C* f) {
@@ -310,7 +322,7 @@ LBPC_HD void gather_f(const Args& a, const NB& b, int n,
             if constexpr (LAYOUT == LAYOUT_PULL) slot = w ? op : q;                      \
             else slot = w ? q : op;                                                     \
         }                                                                               \
-        f[q] = S::dec(ldv<P, LAYOUT, NC>(fs + (size_t)slot * N + idx), fshift(k, q));    \
+        f[q] = S::dec(ldv<P, LAYOUT, HINT>(fs + (size_t)slot * N + idx), fshift(k, q));    \
     }
     LBPC_Q19(LBPC_GF)
 #undef LBPC_GF
@@ -318,7 +330,7 @@ LBPC_HD void gather_f(const Args& a, const NB& b, int n,
 
 // g_1..6 (g[0] is not gathered: the rest population is the FP64 channel h').  The g
 // lattice holds six planes: population q lives in plane q - 1.
-template <int P, int LAYOUT, bool NC, class NB>
+template <int P, int LAYOUT, bool HINT, class NB>
 LBPC_HD void gather_g(const Args& a, const NB& b, int n, int x, int y, int z,
                                          const typename Store<P>::T* gs,
                                          typename Store<P>::C* g) {
@@ -329,15 +341,15 @@ LBPC_HD void gather_g(const Args& a, const NB& b, int n, int x, int y, int z,
 #define LBPC_GG(q, ex, ey, ez, op)                                                       \
     {                                                                                   \
         if constexpr (LAYOUT == LAYOUT_AA_NATURAL) {                                    \
-            g[q] = S::dec(ldv<P, LAYOUT, NC>(gs + (size_t)(q - 1) * N + n), k.gshift);         \
+            g[q] = S::dec(ldv<P, LAYOUT, HINT>(gs + (size_t)(q - 1) * N + n), k.gshift);         \
         } else {                                                                        \
             const bool w = b.template wall<ex, ey, ez>();                                      \
             const int idx = w ? n : n + b.template off<ex, ey, ez>();                          \
             int slot;                                                                   \
             if constexpr (LAYOUT == LAYOUT_PULL) slot = w ? op : q;                      \
             else slot = w ? q : op;                                                     \
-            C v = S::dec(ldv<P, LAYOUT, NC>(gs + (size_t)(slot - 1) * N + idx), k.gshift);     \
-            if (w && a.wall_iso[q - 1]) v = S::grid(-v + abb_source(a, k, q - 1, x, y, z)); \
+            C v = S::dec(ldv<P, LAYOUT, HINT>(gs + (size_t)(slot - 1) * N + idx), k.gshift);     \
+            if (w && a.wall_iso[q - 1]) v = S::grid(abb_back(a, k, q - 1, x, y, z, v));   \
             g[q] = v;                                                                   \
         }                                                                               \
     }
@@ -395,7 +407,7 @@ LBPC_HD void scatter_g(const Args& a, const NB& b, int n, int x, int y, int z,
             if (w) {                                                                    \
                 auto vb = v;                                                            \
                 if (a.wall_iso[op - 1])                                                 \
-                    vb = S::enc_g(-S::dec(v, k.gshift) + abb_source(a, k, op - 1, x, y, z), \
+                    vb = S::enc_g(abb_back(a, k, op - 1, x, y, z, S::dec(v, k.gshift)), \
                                   k.gshift);                                            \
                 gd[(size_t)(op - 1) * N + n] = vb;                                            \
             } else {                                                                    \
@@ -669,23 +681,27 @@ LBPC_HD void collide_flow(C* f, const Coef<C>& k, C T, C fl, C& ux, C& uy, C& uz
 // D3Q7 enthalpy collision on the six moving populations (Eq. 21-25; SRT when every
 // rate equals 1/tau_g).  With d_a = g_a - g_a^eq, d_0 = -sum d_a (h is conserved), the
 // moments of d are m1..m3 (odd pairs), m4 = -7 S, m5, m6; g* = g^eq + d - N^-1 R N d.
-// VAR (conduction kernels): with per-phase conductivities the rates follow from f_l.
-template <class C, bool VAR = false>
+// COND (conduction kernels): u = 0, and with per-phase conductivities the rates follow from
+// f_l.
+template <class C, bool COND = false>
 LBPC_HD void collide_enth(C* g, const Coef<C>& k, C T, C fl, C ux, C uy, C uz) {
-    const C Cp = k.Cps + fl * k.dCp;
     // an axis pair's equilibria (Eq. 7) sum to cT2 (representation) and differ by vT2 u
     const C cT2 = k.wT_cref * T - k.gshift2;
-    const C vT2 = Cp * T;
     // moments of d = g - g^eq: odd pair differences m1..m3, pair sums p
-    const C m1 = (g[1] - g[2]) - vT2 * ux;
-    const C m2 = (g[3] - g[4]) - vT2 * uy;
-    const C m3 = (g[5] - g[6]) - vT2 * uz;
+    C m1 = g[1] - g[2], m2 = g[3] - g[4], m3 = g[5] - g[6];
+    if constexpr (!COND) {
+        const C Cp = k.Cps + fl * k.dCp;
+        const C vT2 = Cp * T;
+        m1 -= vT2 * ux;
+        m2 -= vT2 * uy;
+        m3 -= vT2 * uz;
+    }
     const C p12 = (g[1] + g[2]) - cT2, p34 = (g[3] + g[4]) - cT2, p56 = (g[5] + g[6]) - cT2;
     const C q = p34 + p56;
     const C S = p12 + q, m5 = C(2) * p12 - q, m6 = p34 - p56;
     // g* = g^eq + d - N^-1 R N d = g - N^-1 R N d, rates and 1/|row|^2 folded on the host
     C s46 = k.sig4_6, s56 = k.sig5_6, s64 = k.sig6_4, hchi = k.hchi;
-    if (VAR && k.varchi) {  // Eq. 34 per node, lambda(f_l) linear in f_l
+    if (COND && k.varchi) {  // Eq. 34 per node, lambda(f_l) linear in f_l
         const C sc = C(1) / (k.chi_a + k.chi_b * fl);
         const C s4 = k.s4_a + k.s4_b * sc;
         s46 = s4 * C(1.0 / 6.0);
@@ -724,13 +740,15 @@ LBPC_HD void sum6_pair(const float* g, float& hi, float& lo) {
     two_sum(hi, g[5], hi, e); lo += e;
     two_sum(hi, g[6], hi, e); lo += e;
 }
-// e' + sum g_a and e - sum g_a.  FP64: plain FP64 sums.  FP32 storage: exact FP32 pair
+// e' + sum g_a and e - sum g_a.  FP64: FP64 sums, as trees (a chain of dependent FP64
+// additions is what a conduction step waits for on small lattices; the pair sums are those
+// of the collision).  FP32 storage: exact FP32 pair
 // sums (TwoSum).  16-bit storage: the six values lie on a 2^-20 grid, so a plain FP32
 // sum is already exact.
 template <int P>
 LBPC_HD double excess_plus(double ep, const typename Store<P>::C* g) {
     if constexpr (P == LBPC_FP64) {
-        return ep + g[1] + g[2] + g[3] + g[4] + g[5] + g[6];
+        return ep + (((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]));
     } else if constexpr (Store<P>::kGrid) {
         return ep + f2d_exact(((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]));
     } else {
@@ -742,7 +760,7 @@ LBPC_HD double excess_plus(double ep, const typename Store<P>::C* g) {
 template <int P>
 LBPC_HD double excess_minus(double e, const typename Store<P>::C* g) {
     if constexpr (P == LBPC_FP64) {
-        return e - g[1] - g[2] - g[3] - g[4] - g[5] - g[6];
+        return e - (((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]));
     } else if constexpr (Store<P>::kGrid) {
         return e - f2d_exact(((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]));
     } else {
@@ -755,7 +773,6 @@ LBPC_HD double excess_minus(double e, const typename Store<P>::C* g) {
 // ---------------------------------------------------------------------------------
 // Node-level operations (host + device: the kernels below call them once per node).
 // ---------------------------------------------------------------------------------
-constexpr int STEP_THREADS = 128;
 // Largest lattice the pair paths take: they form plane offsets of up to 3 N in int.
 constexpr int kPairMaxN = 715827882;  // floor((2^31 - 1) / 3)
 
@@ -775,18 +792,18 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     const Coef<C>& k = coef<C>(a);
     const int n = x + a.nx * (y + a.ny * z);
     constexpr int LAYOUT = KindLayout<KIND>::value;
-    constexpr bool NC = KIND == STEP_PULL;  // read-only path only when src != dst
+    constexpr bool HINT = KIND == STEP_PULL;
     const bool interior = is_interior(a, x, y, z);
     const NbInterior bi{a.nx, a.nx * a.ny};
     const Nb b = make_nb(a, x, y, z);
 
     C f[19], g[7];
     if (interior) {
-        if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, NC>(a, bi, n, fs, f);
-        gather_g<Mode<P>::G, LAYOUT, NC>(a, bi, n, x, y, z, gs, g);
+        if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, HINT>(a, bi, n, fs, f);
+        gather_g<Mode<P>::G, LAYOUT, HINT>(a, bi, n, x, y, z, gs, g);
     } else {
-        if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, NC>(a, b, n, fs, f);
-        gather_g<Mode<P>::G, LAYOUT, NC>(a, b, n, x, y, z, gs, g);
+        if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, HINT>(a, b, n, fs, f);
+        gather_g<Mode<P>::G, LAYOUT, HINT>(a, b, n, x, y, z, gs, g);
     }
     const double e = excess_plus<Mode<P>::G>(hp[n], g);  // h - h_s
 
@@ -850,13 +867,14 @@ LBPC_HD void pair_collide(const Args& a, CT<P>* f0, CT<P>* f1, CT<P>* g0, CT<P>*
     collide_enth<C, !FLOW>(g1, k, T1, fl1, ux1, uy1, uz1);
 }
 
-// Two nodes (x0, x0 + 1), x0 even, of a row away from every y and z face: populations
-// with e_x = 0 move as aligned pairs; e_x = +-1 ones are two scalar loads, with the x-face
-// rules (periodic wrap; at a wall the reflected population of the node itself) applied
-// by selecting a 32-bit element offset from the population's plane on the lanes at x = 0
-// / x = nx - 1; every store is a pair.  Requires even nx.
-template <int P, int FLOW, bool TAPE = false>
-LBPC_HD void step_pair_pull(const Args& a, int x0, int y, int z, const TF<P>* fs,
+// Two nodes (x0, x0 + 1), x0 even, of one row: populations with e_x = 0 move as aligned
+// pairs; e_x = +-1 ones are two scalar loads, with the x-face rules (periodic wrap; at a
+// wall the reflected population of the node itself) applied by selecting a 32-bit element
+// offset from the population's plane on the lanes at x = 0 / x = nx - 1; every store is a
+// pair.  The y and z rules are the row's: NbInterior has none (a row away from those
+// faces), Nb selects the wrapped or reflected offset per population.  Requires even nx.
+template <int P, int FLOW, bool TAPE, class NB>
+LBPC_HD void step_pair_pull(const Args& a, const NB& nb, int x0, int y, int z, const TF<P>* fs,
                             TF<P>* fd, const TG<P>* gs,
                             TG<P>* gd, double* hp, CT<P>* tape_e = nullptr,
                             CT<P>* tape_m = nullptr) {
@@ -872,7 +890,6 @@ LBPC_HD void step_pair_pull(const Args& a, int x0, int y, int z, const TF<P>* fs
     const Coef<C>& k = coef<C>(a);
     const size_t N = (size_t)a.N;
     const int N32 = a.N;  // 3 N < 2^31 (kPairMaxN)
-    const int sy = a.nx, sz = a.nx * a.ny;
     const int n0 = x0 + a.nx * (y + a.ny * z), n1 = n0 + 1;
     const bool xlo = x0 == 0, xhi = x0 + 1 == a.nx - 1;
     const bool wlo = xlo && a.wall[0], whi = xhi && a.wall[1];
@@ -880,22 +897,28 @@ LBPC_HD void step_pair_pull(const Args& a, int x0, int y, int z, const TF<P>* fs
     const int up0 = xlo ? n0 + a.nx - 1 : n0 - 1;
     const int up1 = xhi ? n1 - (a.nx - 1) : n1 + 1;
     C f0[19], f1[19], g0[7], g1[7];
+    // 16-bit g: the rest channel first, 0.5-1% of a step; FP32: last, 0.4%
+    constexpr bool EARLY = Store<Mode<P>::G>::kGrid;
+    double2 ep;
+    if constexpr (EARLY) ep = *reinterpret_cast<const double2*>(hp + n0);
     if constexpr (FLOW) {
 #define LBPC_PF(q, ex, ey, ez, op)                                                       \
         {                                                                               \
-            const int oyz = -(ey) * sy - (ez) * sz;                                     \
+            const int oyz = nb.template off<0, ey, ez>();                               \
+            const bool w = nb.template wall<0, ey, ez>();                               \
+            const int ob = ((op) - (q)) * N32;  /* the reflected population's plane */    \
             const C sh = fshift(k, q);                                                  \
             const TFt* pl = fs + (size_t)q * N;                                           \
             if constexpr ((ex) == 0) {                                                  \
-                PRF::dec(ld_any<true>(reinterpret_cast<const VF*>(pl + n0 + oyz)),             \
+                PRF::dec(ld_any<true>(reinterpret_cast<const VF*>(pl + n0 + (w ? ob : oyz))),  \
                         sh, f0[q], f1[q]);                                              \
             } else if constexpr ((ex) == 1) {                                           \
-                const int i0 = wlo ? ((op) - (q)) * N32 + n0 : up0 + oyz;               \
+                const int i0 = w || wlo ? ob + n0 : up0 + oyz;                          \
                 f0[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + i0), sh);                 \
-                f1[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + n0 + oyz), sh);           \
+                f1[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + (w ? ob + n1 : n0 + oyz)), sh); \
             } else {                                                                    \
-                const int i1 = whi ? ((op) - (q)) * N32 + n1 : up1 + oyz;               \
-                f0[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + n1 + oyz), sh);           \
+                const int i1 = w || whi ? ob + n1 : up1 + oyz;                          \
+                f0[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + (w ? ob + n0 : n1 + oyz)), sh); \
                 f1[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + i1), sh);                 \
             }                                                                           \
         }
@@ -904,19 +927,25 @@ LBPC_HD void step_pair_pull(const Args& a, int x0, int y, int z, const TF<P>* fs
     }
 #define LBPC_PG(q, ex, ey, ez, op)                                                       \
     {                                                                                   \
-        const int oyz = -(ey) * sy - (ez) * sz;                                         \
+        const int oyz = nb.template off<0, ey, ez>();                                   \
+        const bool w = nb.template wall<0, ey, ez>();                                   \
+        const int ob = ((op) - (q)) * N32;                                              \
         const TGt* pl = gs + (size_t)(q - 1) * N;                                         \
         if constexpr ((ex) == 0) {                                                      \
-            PRG::dec(ld_any<true>(reinterpret_cast<const VG*>(pl + n0 + oyz)),                 \
+            PRG::dec(ld_any<true>(reinterpret_cast<const VG*>(pl + n0 + (w ? ob : oyz))),      \
                     k.gshift, g0[q], g1[q]);                                            \
+            if (w && a.wall_iso[q - 1]) {                                               \
+                g0[q] = SG::grid(-g0[q] + abb_source(a, k, q - 1, x0, y, z));           \
+                g1[q] = SG::grid(-g1[q] + abb_source(a, k, q - 1, x0 + 1, y, z));       \
+            }                                                                           \
         } else if constexpr ((ex) == 1) {                                               \
-            const int i0 = wlo ? ((op) - (q)) * N32 + n0 : up0 + oyz;                   \
+            const int i0 = wlo ? ob + n0 : up0 + oyz;                                   \
             C v = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + i0), k.gshift);                 \
             if (wlo && a.wall_iso[0]) v = SG::grid(-v + abb_source(a, k, 0, x0, y, z)); \
             g0[q] = v;                                                                  \
             g1[q] = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + n0 + oyz), k.gshift);         \
         } else {                                                                        \
-            const int i1 = whi ? ((op) - (q)) * N32 + n1 : up1 + oyz;                   \
+            const int i1 = whi ? ob + n1 : up1 + oyz;                                   \
             C v = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + i1), k.gshift);                 \
             if (whi && a.wall_iso[1]) v = SG::grid(-v + abb_source(a, k, 1, x0 + 1, y, z)); \
             g1[q] = v;                                                                  \
@@ -925,7 +954,7 @@ LBPC_HD void step_pair_pull(const Args& a, int x0, int y, int z, const TF<P>* fs
     }
     LBPC_Q7(LBPC_PG)
 #undef LBPC_PG
-    const double2 ep = ld_any<true>(reinterpret_cast<const double2*>(hp + n0));
+    if constexpr (!EARLY) ep = *reinterpret_cast<const double2*>(hp + n0);
     const double e0 = excess_plus<Mode<P>::G>(ep.x, g0), e1 = excess_plus<Mode<P>::G>(ep.y, g1);
     pair_collide<P, FLOW, TAPE>(a, f0, f1, g0, g1, e0, e1, n0, tape_e, tape_m);
     if constexpr (FLOW) {
@@ -1553,11 +1582,11 @@ LBPC_HD CT<P> adj_reverse_node(const Args& a, const NB& b, int x, int y, int z,
     return dL;
 }
 
-// Reverse step of two nodes (x0, x0 + 1) of a row away from every y and z face (even nx):
+// Reverse step of two nodes (x0, x0 + 1) of one row (even nx; NB: the row's y and z rules):
 // lambda_q of node x is lambda_{n+1} in plane q at x + e_q, or the reflected plane at x
-// when x + e_q lies behind an x wall; every other access is an aligned pair.
-template <int P, bool FLOW>
-LBPC_HD CT<P> adj_reverse_pair(const Args& a, int x0, int y, int z, const CT<P>* lin,
+// when x + e_q lies behind a wall; e_x = 0 accesses are aligned pairs.
+template <int P, bool FLOW, class NB>
+LBPC_HD CT<P> adj_reverse_pair(const Args& a, const NB& nb, int x0, int y, int z, const CT<P>* lin,
                                CT<P>* lout, const CT<P>* tape_e, const CT<P>* tape_m,
                                int wface, double* gtw) {
     using C = CT<P>;
@@ -1566,7 +1595,6 @@ LBPC_HD CT<P> adj_reverse_pair(const Args& a, int x0, int y, int z, const CT<P>*
     const size_t N = (size_t)a.N;
     const int N32 = a.N;  // 3 N < 2^31 (kPairMaxN)
     constexpr int nf = FLOW ? 19 : 0;
-    const int sy = a.nx, sz = a.nx * a.ny;
     const int n0 = x0 + a.nx * (y + a.ny * z), n1 = n0 + 1;
     const bool xlo = x0 == 0, xhi = x0 + 1 == a.nx - 1;
     const bool wlo = xlo && a.wall[0], whi = xhi && a.wall[1];
@@ -1576,17 +1604,19 @@ LBPC_HD CT<P> adj_reverse_pair(const Args& a, int x0, int y, int z, const CT<P>*
     if constexpr (FLOW) {
 #define LBPC_RF(q, ex, ey, ez, op)                                                       \
         {                                                                               \
-            const int o = (ey) * sy + (ez) * sz;                                        \
+            const int o = nb.template off<0, -(ey), -(ez)>();                           \
+            const bool w = nb.template wall<0, -(ey), -(ez)>();                         \
+            const int ob = ((op) - (q)) * N32;  /* the reflected plane */                 \
             const C* pl = lin + (size_t)q * N;                                          \
             if constexpr ((ex) == 0) {                                                  \
-                const VC v = ld_any<true>(reinterpret_cast<const VC*>(pl + n0 + o));    \
+                const VC v = ld_any<true>(reinterpret_cast<const VC*>(pl + n0 + (w ? ob : o))); \
                 lf0[q] = v.x; lf1[q] = v.y;                                             \
             } else if constexpr ((ex) == 1) {                                           \
-                lf0[q] = ld_any<true>(pl + n1 + o);                                     \
-                lf1[q] = ld_any<true>(pl + (whi ? ((op) - (q)) * N32 + n1 : up1 + o)); \
+                lf0[q] = ld_any<true>(pl + (w ? ob + n0 : n1 + o));                     \
+                lf1[q] = ld_any<true>(pl + (w || whi ? ob + n1 : up1 + o));             \
             } else {                                                                    \
-                lf0[q] = ld_any<true>(pl + (wlo ? ((op) - (q)) * N32 + n0 : dn0 + o)); \
-                lf1[q] = ld_any<true>(pl + n0 + o);                                     \
+                lf0[q] = ld_any<true>(pl + (w || wlo ? ob + n0 : dn0 + o));             \
+                lf1[q] = ld_any<true>(pl + (w ? ob + n1 : n0 + o));                     \
             }                                                                           \
         }
         LBPC_Q19(LBPC_RF)
@@ -1598,19 +1628,27 @@ LBPC_HD CT<P> adj_reverse_pair(const Args& a, int x0, int y, int z, const CT<P>*
     }
 #define LBPC_RG(q, ex, ey, ez, op)                                                       \
     {                                                                                   \
-        const int o = (ey) * sy + (ez) * sz;                                            \
+        const int o = nb.template off<0, -(ey), -(ez)>();                               \
+        const bool w = nb.template wall<0, -(ey), -(ez)>();                             \
+        const int ob = ((op) - (q)) * N32;                                              \
         const C* pl = lin + (size_t)(nf + q) * N;                                       \
         if constexpr ((ex) == 0) {                                                      \
-            const VC v = ld_any<true>(reinterpret_cast<const VC*>(pl + n0 + o));        \
-            lg0[q] = v.x; lg1[q] = v.y;                                                 \
+            const VC v = ld_any<true>(reinterpret_cast<const VC*>(pl + n0 + (w ? ob : o))); \
+            const bool iso = w && a.wall_iso[op - 1];                                   \
+            lg0[q] = iso ? -v.x : v.x;                                                  \
+            lg1[q] = iso ? -v.y : v.y;                                                  \
+            if (iso && wface == op - 1) {                                               \
+                gtw[face_index(a, op - 1, x0, y, z)] += wall_grad(k, v.x);              \
+                gtw[face_index(a, op - 1, x0 + 1, y, z)] += wall_grad(k, v.y);          \
+            }                                                                           \
         } else if constexpr ((ex) == 1) {                                               \
             lg0[q] = ld_any<true>(pl + n1 + o);                                         \
-            const C la = ld_any<true>(pl + (whi ? ((op) - (q)) * N32 + n1 : up1 + o));  \
+            const C la = ld_any<true>(pl + (whi ? ob + n1 : up1 + o));                \
             const bool iso = whi && a.wall_iso[1];                                      \
             lg1[q] = iso ? -la : la;                                                    \
             if (iso && wface == 1) gtw[y + a.ny * z] += wall_grad(k, la);          \
         } else {                                                                        \
-            const C la = ld_any<true>(pl + (wlo ? ((op) - (q)) * N32 + n0 : dn0 + o));  \
+            const C la = ld_any<true>(pl + (wlo ? ob + n0 : dn0 + o));                \
             const bool iso = wlo && a.wall_iso[0];                                      \
             lg0[q] = iso ? -la : la;                                                    \
             if (iso && wface == 0) gtw[y + a.ny * z] += wall_grad(k, la);          \
@@ -1642,13 +1680,54 @@ LBPC_HD CT<P> adj_reverse_pair(const Args& a, int x0, int y, int z, const CT<P>*
 
 #if defined(__CUDACC__)
 // ---------------------------------------------------------------------------------
-// Kernels: one thread per node on a (x-block, y-block, z) grid.
+// Kernels: one thread per node or node pair, on the grid of item_grid().
 // ---------------------------------------------------------------------------------
+// Column (node or pair) c, y and z of this thread's item in a lattice of cols x ny x nz
+// items.  Row lengths that fill whole blocks take the grid's own coordinates (the division
+// below costs 2% of a 16-bit step); for the others threads count the items in memory order, so
+// that a warp runs on across row ends instead of idling there (of 80 or 96 columns, 64-wide
+// blocks idled 37% or 25%: the 16-bit step of 160 x 160 x 80 took 62 us, now 48).  gridDim.y =
+// nz: each z plane has its own blocks; otherwise one run over the whole lattice.
+__device__ __forceinline__ bool item_cyz(const Args& a, int cols, const FastDiv& by_cols, int fill,
+                                         int& c, int& y, int& z) {
+    if (fill) {
+        c = blockIdx.x * blockDim.x + threadIdx.x;
+        y = blockIdx.y * blockDim.y + threadIdx.y;
+        z = blockIdx.z;
+        return y < a.ny;
+    }
+    const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned row = by_cols.div(p);
+    c = (int)(p - row * (unsigned)cols);
+    if (gridDim.y == 1) {
+        z = (int)a.by_ny.div(row);
+        y = (int)row - z * a.ny;
+        return z < a.nz;
+    }
+    z = blockIdx.y;
+    y = (int)row;
+    return y < a.ny;
+}
+
+// In the kernels that follow one another step by step, before any access to their data: lets
+// the next grid of the stream become resident while this one drains, then waits until the
+// previous grid has completed and its stores are visible.  The pointers given go through the
+// barrier: for data that the kernel only reads (const __restrict__) so that no load of it,
+// which the compiler may take for a constant, is moved above; in the pair kernels because the
+// compiler then forms addresses from them after it (which ones is a measurement: up to 8% of a
+// 16-bit step either way).
+// Why: between two dependent launches the GPU waits in steps of about 2 us; 64^3 FP32 took
+// 10.3 us a step without the overlap and 8.0 us with it (6.2 -> 3.1 us at 64 x 1 x 64).
+template <class... Ptr>
+__device__ __forceinline__ void after_previous_grid(Ptr&... p) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (opaque(p), ...);
+}
+
 #define LBPC_NODE_XYZ                                                                    \
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;                                \
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;                                \
-    const int z = blockIdx.z;                                                           \
-    if (x >= a.nx || y >= a.ny) return;
+    int x, y, z;                                                                        \
+    if (!item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z)) return;
 
 // One node per thread; with TAPE (pull) also the adjoint tape.
 template <int P, int KIND, int FLOW, bool TAPE>
@@ -1656,36 +1735,57 @@ __global__ void __launch_bounds__(STEP_THREADS)
 k_step(const __grid_constant__ Args a, const TF<P>* fs, TF<P>* fd,
        const TG<P>* gs, TG<P>* gd, double* __restrict__ hp, CT<P>* __restrict__ tape_e,
        CT<P>* __restrict__ tape_m) {
-    LBPC_NODE_XYZ
+    int x, y, z;
+    const bool valid = item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z);
+    after_previous_grid(fs, fd, gs, gd, hp);
+    if (!valid) return;
     step_node<P, KIND, FLOW, TAPE>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
 }
 
 
-// Pull step, two nodes per thread along x (even nx).  Warps whose rows all lie away
-// from the y and z faces take the paired path; others run the per-node path twice.
+// Pull step, two nodes per thread along x (even nx).  Warps whose rows all lie away from
+// the y and z faces take the path without those faces' rules.
 // With TAPE also the adjoint tape.  Blocks per SM: FP32 five (96 registers), four when
-// taping; 16-bit f (collision rebuilt from the moments) six (80 registers), five when taping.
+// taping; 16-bit f and g (collision rebuilt from the moments) six (80 registers), five when
+// taping; 16-bit f with FP32 g five (256 x 256 x 128: 188 us a step at five, 191 FP16 / 212
+// BF16 at six).
+template <int P>
+constexpr int kPullBlocks = sizeof(TG<P>) == 2 ? 6 : 5;
 template <int P, int FLOW, bool TAPE>
-__global__ void __launch_bounds__(STEP_THREADS, TAPE ? (kRebuild<P> ? 5 : 4) : (kRebuild<P> ? 6 : 5))
+__global__ void __launch_bounds__(STEP_THREADS, TAPE ? (kRebuild<P> ? 5 : 4) : kPullBlocks<P>)
 k_step_pull_x2(const __grid_constant__ Args a, const TF<P>* fs,
                TF<P>* fd, const TG<P>* gs, TG<P>* gd,
                double* __restrict__ hp, CT<P>* __restrict__ tape_e,
                CT<P>* __restrict__ tape_m) {
-    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    const bool valid = x0 < a.nx && y < a.ny;
+    int x0, y, z;
+    const bool valid = item_cyz(a, a.nx / 2, a.by_hx, a.fill_hx, x0, y, z);
+    x0 *= 2;
     const bool inner = !valid || (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1);
-    const bool paired = __all_sync(0xffffffffu, inner);
+    const bool plain = __all_sync(0xffffffffu, inner);
+    after_previous_grid(fd, gd, hp);
     if (!valid) return;
-    if (paired) {
-        step_pair_pull<P, FLOW, TAPE>(a, x0, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
+    if (plain) {
+        step_pair_pull<P, FLOW, TAPE>(a, NbInterior{a.nx, a.nx * a.ny}, x0, y, z, fs, fd, gs, gd,
+                                      hp, tape_e, tape_m);
     } else {
-        step_node<P, STEP_PULL, FLOW, TAPE>(a, x0, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
-        step_node<P, STEP_PULL, FLOW, TAPE>(a, x0 + 1, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
+        step_pair_pull<P, FLOW, TAPE>(a, make_nb(a, x0, y, z), x0, y, z, fs, fd, gs, gd, hp,
+                                      tape_e, tape_m);
     }
 }
 
+
+// The face rows of an AA step.  With 16-bit f and FP32 g kept out of line: inlined, they cost
+// the interior path 4% (its registers).
+template <int P, int KIND, int FLOW>
+LBPC_HD void aa_face_pair(const Args& a, int x0, int y, int z, TF<P>* F, TG<P>* G, double* hp) {
+    step_node<P, KIND, FLOW>(a, x0, y, z, F, F, G, G, hp);
+    step_node<P, KIND, FLOW>(a, x0 + 1, y, z, F, F, G, G, hp);
+}
+template <int P, int KIND, int FLOW>
+__device__ __noinline__ void aa_face_pair_call(const Args& a, int x0, int y, int z, TF<P>* F,
+                                               TG<P>* G, double* hp) {
+    aa_face_pair<P, KIND, FLOW>(a, x0, y, z, F, G, hp);
+}
 
 // AA step, two nodes per thread along x (even nx); same vote as the pull pair kernel.
 // Five blocks per SM (96 registers; a few bytes of spills in some variants); the even step
@@ -1693,19 +1793,21 @@ k_step_pull_x2(const __grid_constant__ Args a, const TF<P>* fs,
 template <int P, int FLOW, bool ODD>
 __global__ void __launch_bounds__(STEP_THREADS, kRebuild<P> && !ODD ? 6 : 5)
 k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* __restrict__ hp) {
-    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    const bool valid = x0 < a.nx && y < a.ny;
+    int x0, y, z;
+    const bool valid = item_cyz(a, a.nx / 2, a.by_hx, a.fill_hx, x0, y, z);
+    x0 *= 2;
     const bool inner = !valid || (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1);
     const bool paired = __all_sync(0xffffffffu, inner);
+    constexpr bool MIXED = kRebuild<P> && sizeof(TG<P>) == 4;
+    if constexpr (MIXED) after_previous_grid(hp);
+    else after_previous_grid(F, G);
     if (!valid) return;
     constexpr int KIND = ODD ? STEP_AA_ODD : STEP_AA_EVEN;
     if (paired) {
         step_pair_aa<P, FLOW, ODD>(a, x0, y, z, F, G, hp);
     } else {
-        step_node<P, KIND, FLOW>(a, x0, y, z, F, F, G, G, hp);
-        step_node<P, KIND, FLOW>(a, x0 + 1, y, z, F, F, G, G, hp);
+        if constexpr (MIXED) aa_face_pair_call<P, KIND, FLOW>(a, x0, y, z, F, G, hp);
+        else aa_face_pair<P, KIND, FLOW>(a, x0, y, z, F, G, hp);
     }
 }
 
@@ -1803,11 +1905,13 @@ k_check(const __grid_constant__ Args a, const TG<P>* __restrict__ g,
 }
 
 // ---- adjoint kernels ----
+__device__ __forceinline__ int block_thread() { return threadIdx.x + blockDim.x * threadIdx.y; }
+
 // Sum of v over the block (STEP_THREADS threads), valid in thread 0.
 __device__ __forceinline__ double block_sum(double v) {
     __shared__ double sh[STEP_THREADS / 32];
     v = warp_sum(v);
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
+    const int tid = block_thread();
     if ((tid & 31) == 0) sh[tid >> 5] = v;
     __syncthreads();
     double s = 0.0;
@@ -1820,10 +1924,9 @@ __device__ __forceinline__ int block_linear() {
     return blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
 }
 
-// Per-warp slot of the adjoint's dJ/dL partials (ADJ_WARPS_PER_BLOCK per block).
-static_assert(STEP_THREADS / 32 == ADJ_WARPS_PER_BLOCK, "one partial slot per warp");
+// Per-warp slot of the adjoint's dJ/dL partials.
 __device__ __forceinline__ int warp_slot() {
-    return block_linear() * ADJ_WARPS_PER_BLOCK + ((threadIdx.x + blockDim.x * threadIdx.y) >> 5);
+    return block_linear() * (STEP_THREADS / 32) + (block_thread() >> 5);
 }
 
 template <int P, bool FLOW>
@@ -1831,15 +1934,13 @@ __global__ void __launch_bounds__(STEP_THREADS)
 k_adj_seed(const __grid_constant__ Args a, const TG<P>* __restrict__ gs,
            const double* __restrict__ hp, CT<P>* __restrict__ lam,
            double* __restrict__ Lpart, double* __restrict__ Jpart) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
+    int x, y, z;
     double dL = 0.0, fl = 0.0;
-    if (x < a.nx && y < a.ny) dL = (double)adj_seed_node<P, FLOW>(a, x, y, z, gs, hp, lam, fl);
+    if (item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z)) dL = (double)adj_seed_node<P, FLOW>(a, x, y, z, gs, hp, lam, fl);
     const double wL = warp_sum(dL);
-    if (((threadIdx.x + blockDim.x * threadIdx.y) & 31) == 0) Lpart[warp_slot()] = wL;
+    if ((block_thread() & 31) == 0) Lpart[warp_slot()] = wL;
     const double sJ = block_sum(fl);
-    if (threadIdx.x == 0 && threadIdx.y == 0) Jpart[block_linear()] = sJ;
+    if (block_thread() == 0) Jpart[block_linear()] = sJ;
 }
 
 template <int P, bool FLOW>
@@ -1848,11 +1949,11 @@ k_adj_reverse(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
               CT<P>* __restrict__ lout, const CT<P>* __restrict__ tape_e,
               const CT<P>* __restrict__ tape_m, int wface, double* gtw,
               double* __restrict__ Lpart) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
+    int x, y, z;
     CT<P> dL = CT<P>(0);
-    if (x < a.nx && y < a.ny) {
+    const bool valid = item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z);
+    after_previous_grid(lin, tape_e, tape_m);
+    if (valid) {
         if (is_interior(a, x, y, z))
             dL = adj_reverse_node<P, FLOW>(a, NbInterior{a.nx, a.nx * a.ny}, x, y, z, lin, lout,
                                            tape_e, tape_m, wface, gtw);
@@ -1863,7 +1964,7 @@ k_adj_reverse(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
     // warp partials only (no block barrier in the reverse sweep), summed within the warp in
     // the compute precision and accumulated over warps and steps in FP64
     const CT<P> w = warp_sum(dL);
-    if (((threadIdx.x + blockDim.x * threadIdx.y) & 31) == 0) Lpart[warp_slot()] += (double)w;
+    if ((block_thread() & 31) == 0) Lpart[warp_slot()] += (double)w;
 }
 
 // Reverse step, two nodes per thread along x (even nx); the pull kernels' vote.  Five
@@ -1874,34 +1975,54 @@ k_adj_reverse_x2(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
                  CT<P>* __restrict__ lout, const CT<P>* __restrict__ tape_e,
                  const CT<P>* __restrict__ tape_m, int wface, double* gtw,
                  double* __restrict__ Lpart) {
-    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    const bool valid = x0 < a.nx && y < a.ny;
+    int x0, y, z;
+    const bool valid = item_cyz(a, a.nx / 2, a.by_hx, a.fill_hx, x0, y, z);
+    x0 *= 2;
     const bool inner = !valid || (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1);
-    const bool paired = __all_sync(0xffffffffu, inner);
+    const bool plain = __all_sync(0xffffffffu, inner);
     CT<P> dL = CT<P>(0);
+    after_previous_grid(lin, tape_e, tape_m);
     if (valid) {
-        if (paired) {
-            dL = adj_reverse_pair<P, FLOW>(a, x0, y, z, lin, lout, tape_e, tape_m, wface, gtw);
-        } else {
-            for (int x = x0; x < x0 + 2; x++)
-                dL += adj_reverse_node<P, FLOW>(a, make_nb(a, x, y, z), x, y, z, lin, lout, tape_e,
-                                                tape_m, wface, gtw);
-        }
+        if (plain)
+            dL = adj_reverse_pair<P, FLOW>(a, NbInterior{a.nx, a.nx * a.ny}, x0, y, z, lin, lout,
+                                           tape_e, tape_m, wface, gtw);
+        else
+            dL = adj_reverse_pair<P, FLOW>(a, make_nb(a, x0, y, z), x0, y, z, lin, lout, tape_e,
+                                           tape_m, wface, gtw);
     }
     // warp partials in the compute precision, accumulated in FP64 (see k_adj_reverse)
     const CT<P> w = warp_sum(dL);
-    if (((threadIdx.x + blockDim.x * threadIdx.y) & 31) == 0) Lpart[warp_slot()] += (double)w;
+    if ((block_thread() & 31) == 0) Lpart[warp_slot()] += (double)w;
 }
 
 // ---------------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------------
-inline dim3 node_block(const Args& a) { return node_block_dims(a.nx); }
-inline dim3 node_grid(const Args& a, dim3 blk) {
-    return dim3((a.nx + blk.x - 1) / blk.x, (a.ny + blk.y - 1) / blk.y, a.nz);
+// Launch of a kernel that begins with after_previous_grid(): with `early` its blocks may
+// become resident before the stream's previous kernel has completed.
+template <class... K, class... A>
+inline void launch_after(void (*kern)(K...), const ItemGrid& g, bool early, cudaStream_t s,
+                         A... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = g.grid;
+    c.blockDim = g.block;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&c, kern, K(args)...);
 }
+// FP64 grids between one warp and six blocks per SM start after the one before instead: early
+// blocks go where that one left room, two to an SM beside idle ones, and share its FP64 pipe
+// (24^3 flow: 35 us a step early, 14.5 after; 8 x 8 x 64: 11.4 and 12.5; 64^3: 153 and 156).
+template <int P>
+inline bool start_early(const Args& a) {
+    return P != LBPC_FP64 || a.N <= SM_COUNT * 32 || a.N >= 6 * SM_COUNT * STEP_THREADS;
+}
+inline ItemGrid node_grid(const Args& a) { return item_grid(a.nx, a.ny, a.nz); }
+inline ItemGrid pair_grid(const Args& a) { return item_grid(a.nx / 2, a.ny, a.nz); }
 
 template <int P>
 struct Impl {
@@ -1916,22 +2037,17 @@ struct Impl {
         using C = CT<P>;
         if constexpr (P != LBPC_FP64) {  // FP64 keeps one node per thread
             if (a.nx % 2 == 0 && a.N <= kPairMaxN) {
-                const int pairs = a.nx / 2;
-                const dim3 blk = node_block_dims(pairs);
-                const dim3 grd((pairs + blk.x - 1) / blk.x, (a.ny + blk.y - 1) / blk.y, a.nz);
                 if constexpr (KIND == STEP_PULL)
-                    k_step_pull_x2<P, FLOW, TAPE><<<grd, blk, 0, s>>>(a, (const T*)fs, (T*)fd,
-                                                                (const TGp*)gs, (TGp*)gd, hp,
-                                                                (C*)tape_e, (C*)tape_m);
+                    launch_after(k_step_pull_x2<P, FLOW, TAPE>, pair_grid(a), true, s, a, (const T*)fs,
+                                 (T*)fd, (const TGp*)gs, (TGp*)gd, hp, (C*)tape_e, (C*)tape_m);
                 else
-                    k_step_aa_x2<P, FLOW, KIND == STEP_AA_ODD><<<grd, blk, 0, s>>>(a, (T*)fd,
-                                                                               (TGp*)gd, hp);
+                    launch_after(k_step_aa_x2<P, FLOW, KIND == STEP_AA_ODD>, pair_grid(a), true, s, a,
+                                 (T*)fd, (TGp*)gd, hp);
                 return;
             }
         }
-        const dim3 blk = node_block(a), grd = node_grid(a, blk);
-        k_step<P, KIND, FLOW, TAPE><<<grd, blk, 0, s>>>(a, (const T*)fs, (T*)fd, (const TGp*)gs, (TGp*)gd, hp,
-                                                  (C*)tape_e, (C*)tape_m);
+        launch_after(k_step<P, KIND, FLOW, TAPE>, node_grid(a), start_early<P>(a), s, a, (const T*)fs, (T*)fd,
+                     (const TGp*)gs, (TGp*)gd, hp, (C*)tape_e, (C*)tape_m);
     }
     static void step(const Args& a, StepKind kind, const void* fs, void* fd, const void* gs,
                      void* gd, double* hp, cudaStream_t s) {
@@ -1972,7 +2088,7 @@ struct Impl {
 
     static void init(const Args& a, Layout lay, const double* Qf, const double* Qg,
                      const double* h0, void* f, void* g, double* hp, cudaStream_t s) {
-        const dim3 blk = node_block(a), grd = node_grid(a, blk);
+        const auto [grd, blk] = node_grid(a);
         if (lay == LAYOUT_PULL) {
             if (a.flow) k_init<P, LAYOUT_PULL, true><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g);
             else k_init<P, LAYOUT_PULL, false><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g);
@@ -1987,7 +2103,7 @@ struct Impl {
     template <int LAYOUT>
     static void dist_k(const Args& a, const void* f, const void* g, const double* hp,
                        double* Qf, double* Qg, cudaStream_t s) {
-        const dim3 blk = node_block(a), grd = node_grid(a, blk);
+        const auto [grd, blk] = node_grid(a);
         if (a.flow) k_dist<P, LAYOUT, true><<<grd, blk, 0, s>>>(a, (const T*)f, (const TGp*)g, hp, Qf, Qg);
         else k_dist<P, LAYOUT, false><<<grd, blk, 0, s>>>(a, (const T*)f, (const TGp*)g, hp, Qf, Qg);
     }
@@ -2009,7 +2125,7 @@ struct Impl {
     }
     static void adj_seed(const Args& a, const void* gs, const double* hp, void* lam,
                          double* Lpart, double* Jpart, cudaStream_t s) {
-        const dim3 blk = node_block(a), grd = node_grid(a, blk);
+        const auto [grd, blk] = node_grid(a);
         using C = CT<P>;
         if (a.flow) k_adj_seed<P, true><<<grd, blk, 0, s>>>(a, (const TGp*)gs, hp, (C*)lam, Lpart, Jpart);
         else k_adj_seed<P, false><<<grd, blk, 0, s>>>(a, (const TGp*)gs, hp, (C*)lam, Lpart, Jpart);
@@ -2019,30 +2135,17 @@ struct Impl {
                             cudaStream_t s) {
         using C = CT<P>;
         if constexpr (P != LBPC_FP64) {
-            // the paired grid never has more blocks than the per-node one that sized Lpart
+            // the paired grid never has more warps than the per-node one that sized Lpart
             if (a.nx % 2 == 0 && a.N <= kPairMaxN) {
-                const int pairs = a.nx / 2;
-                const dim3 blk = node_block_dims(pairs);
-                const dim3 grd((pairs + blk.x - 1) / blk.x, (a.ny + blk.y - 1) / blk.y, a.nz);
-                if (a.flow)
-                    k_adj_reverse_x2<P, true><<<grd, blk, 0, s>>>(a, (const C*)lin, (C*)lout,
-                                                                 (const C*)tape_e, (const C*)tape_m,
-                                                                 wface, gtw, Lpart);
-                else
-                    k_adj_reverse_x2<P, false><<<grd, blk, 0, s>>>(a, (const C*)lin, (C*)lout,
-                                                                  (const C*)tape_e,
-                                                                  (const C*)tape_m, wface, gtw,
-                                                                  Lpart);
+                launch_after(a.flow ? k_adj_reverse_x2<P, true> : k_adj_reverse_x2<P, false>,
+                             pair_grid(a), true, s, a, (const C*)lin, (C*)lout, (const C*)tape_e,
+                             (const C*)tape_m, wface, gtw, Lpart);
                 return;
             }
         }
-        const dim3 blk = node_block(a), grd = node_grid(a, blk);
-        if (a.flow)
-            k_adj_reverse<P, true><<<grd, blk, 0, s>>>(a, (const C*)lin, (C*)lout, (const C*)tape_e,
-                                                       (const C*)tape_m, wface, gtw, Lpart);
-        else
-            k_adj_reverse<P, false><<<grd, blk, 0, s>>>(a, (const C*)lin, (C*)lout, (const C*)tape_e,
-                                                        (const C*)tape_m, wface, gtw, Lpart);
+        launch_after(a.flow ? k_adj_reverse<P, true> : k_adj_reverse<P, false>, node_grid(a), start_early<P>(a), s, a,
+                     (const C*)lin, (C*)lout, (const C*)tape_e, (const C*)tape_m, wface, gtw,
+                     Lpart);
     }
 
     static void check(const Args& a, const void* g, const double* hp, int* flag,
