@@ -25,6 +25,8 @@ struct WsLayout {
     size_t f[2], g[2], hp, tw[6], partial, lines, result, hist, stage, flag, total;
 };
 
+constexpr int CLUSTER_STEPS = 2048;  // steps of one launch on a small lattice, at most
+constexpr int CLUSTER_LEAST = 4;     // and at least: the launch costs about two single steps
 constexpr size_t kAlign = 256;
 constexpr uint32_t kStateMagic = 0x4c425043u;  // "LBPC"
 
@@ -160,6 +162,7 @@ struct lbpc_handle {
     void *f[2], *g[2];
     double *hp, *tw[6], *partial, *lines, *result, *hist, *stage;
     int* flag;
+    bool cluster;  // the lattice is small enough for blocks of steps in one launch
     int cur;
     long long step;
     long long hist_count;
@@ -344,7 +347,10 @@ lbpc_status lbpc_create(int nx, int ny, int nz, const lbpc_params* p, void* dev_
             }
         }
     }
-    if (s == LBPC_OK) s = reset_from_h(h, nullptr);
+    if (s == LBPC_OK) {
+        h->cluster = h->L->cluster_fits(h->args, p->streaming == LBPC_AA);
+        s = reset_from_h(h, nullptr);
+    }
     if (s != LBPC_OK) {
         g_create_err = h->err;
         delete h;
@@ -380,8 +386,19 @@ lbpc_status lbpc_step(lbpc_handle* h, int n) {
     if (s != LBPC_OK) return s;
     const int rep = h->p.report_every;
     bool recorded = false;  // diagnostics taken during this call
-    for (int i = 0; i < n; i++) {
-        if (h->p.streaming == LBPC_PULL) {
+    for (int i = 0; i < n;) {
+        // steps up to the next diagnostics point in one launch (bounded, so that no launch
+        // runs for more than some milliseconds)
+        int take = h->cluster ? std::min(n - i, CLUSTER_STEPS) : 1;
+        if (rep > 0) take = (int)std::min<long long>(take, rep - h->step % rep);
+        if (take < CLUSTER_LEAST) take = 1;
+        if (take > 1) {
+            const bool aa = h->p.streaming == LBPC_AA;
+            const int nb = aa ? h->cur : 1 - h->cur;
+            LBPC_CK(h, h->L->cluster_steps(h->args, aa, h->f[h->cur], h->f[nb], h->g[h->cur],
+                                           h->g[nb], h->hp, take, (int)(h->step % 2), h->stream));
+            h->cur = nb;
+        } else if (h->p.streaming == LBPC_PULL) {
             h->L->step(h->args, STEP_PULL, h->f[h->cur], h->f[1 - h->cur], h->g[h->cur],
                        h->g[1 - h->cur], h->hp, h->stream);
             h->cur = 1 - h->cur;
@@ -389,7 +406,8 @@ lbpc_status lbpc_step(lbpc_handle* h, int n) {
             const StepKind k = (h->step % 2 == 0) ? STEP_AA_EVEN : STEP_AA_ODD;
             h->L->step(h->args, k, h->f[0], h->f[0], h->g[0], h->g[0], h->hp, h->stream);
         }
-        h->step++;
+        i += take;
+        h->step += take;
         h->launches++;
         if (rep > 0 && h->step % rep == 0) {
             s = diagnostics(h, true);

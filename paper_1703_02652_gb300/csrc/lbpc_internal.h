@@ -101,6 +101,11 @@ constexpr int RED_THREADS = 256;
 struct Launchers {
     void (*step)(const Args&, StepKind, const void* fs, void* fd, const void* gs, void* gd,
                  double* hp, cudaStream_t);
+    // small lattices: whether n steps can run on one cluster in one launch, and that launch
+    // (pull: from fs, gs to fd, gd; AA: in place, odd = parity of the first step)
+    bool (*cluster_fits)(const Args&, bool aa);
+    cudaError_t (*cluster_steps)(const Args&, bool aa, const void* fs, void* fd, const void* gs,
+                                 void* gd, double* hp, int n, int odd, cudaStream_t);
     void (*macro)(const Args&, Layout, const void* f, const void* g, const double* hp,
                   const MacroOut&, cudaStream_t);
     // write populations from a pre-collision state Q (f: 19N FP64 or null = rest

@@ -1811,6 +1811,176 @@ k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* __restr
     }
 }
 
+// ---------------------------------------------------------------------------------
+// Small lattices: a block of steps in one launch.
+//
+// A lattice of a few thousand nodes is bound by latency: one launch per step costs 3-4 us
+// even with its start overlapped, most of it the way to the L2 and back.  One cluster of
+// CL_CTAS CTAs keeps the whole lattice on chip instead: thread l of CTA c owns node
+// c * per + l for all n steps, its rest channel stays in a register, and the populations go
+// through two buffers in the CTAs' shared memory (stored precision, so that every rounding
+// is the one of the step-by-step path), read by the downwind neighbours over distributed
+// shared memory.  One hardware cluster barrier per step orders the exchange: step i writes
+// buffer i % 2, which the step before it read and every CTA has since left.  The first
+// gather and the last scatter are the per-node path's, in the layout that the handle holds.
+// Measured, us a step before and after: 64 x 1 x 64 FP32 3.4 and 1.1, 64 x 4 x 4 FP64
+// conduction 3.7 and 2.3, 57 x 1 x 92 FP32 3.4 and 1.4.
+// ---------------------------------------------------------------------------------
+constexpr int CL_CTAS = 16;      // one GPC; more than 8 needs the non-portable attribute
+// nodes of a CTA at most: the lattice sizes up to which the cluster beats the step-by-step
+// path (3-4 us a step, spread over all SMs).  FP64 collisions are bound by the FP64 pipe of
+// the 16 SMs.
+template <int P, bool FLOW>
+constexpr int CL_THREADS = P != LBPC_FP64 ? 512 : (FLOW ? 32 : 256);
+
+__device__ __forceinline__ unsigned shared_at(const void* p, unsigned cta) {
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(cta));
+    return r;
+}
+template <class T>
+__device__ __forceinline__ T ld_cluster(unsigned a) {
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long v;
+        asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a));
+        return *reinterpret_cast<T*>(&v);
+    } else if constexpr (sizeof(T) == 4) {
+        unsigned v;
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a));
+        return *reinterpret_cast<T*>(&v);
+    } else {
+        unsigned short v;
+        asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(a));
+        return *reinterpret_cast<T*>(&v);
+    }
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// n >= 1 steps; odd: parity of the first one (AA only).
+template <int P, bool FLOW, bool AA>
+__global__ void __launch_bounds__(CL_THREADS<P, FLOW>)
+k_steps_cluster(const __grid_constant__ Args a, const TF<P>* fs, TF<P>* fd, const TG<P>* gs,
+                TG<P>* gd, double* hp, int n, int odd, int per) {
+    using SF = Store<Mode<P>::F>;
+    using SG = Store<Mode<P>::G>;
+    using TFt = TF<P>;
+    using TGt = TG<P>;
+    using C = CT<P>;
+    extern __shared__ __align__(16) unsigned char sm[];
+    const Coef<C>& k = coef<C>(a);
+    const int l = threadIdx.x, node = (int)blockIdx.x * per + l;
+    const bool own = l < per && node < a.N;
+    after_previous_grid();
+
+    // [buffer][plane][per]: 19 planes of f (FLOW), then 6 of g
+    const unsigned gbase = FLOW ? 2u * 19u * (unsigned)sizeof(TFt) * (unsigned)per : 0u;
+    const unsigned fhalf = 19u * (unsigned)sizeof(TFt) * (unsigned)per;
+    const unsigned ghalf = 6u * (unsigned)sizeof(TGt) * (unsigned)per;
+    unsigned af[19], ag[7];  // where the upwind population lies (buffer 0)
+    C src[7];                // anti-bounce-back sources (FP64: wall temperatures)
+    unsigned iso = 0;        // bit q: population q comes back from an isothermal wall
+    C f[19], g[7];
+    double ep = 0.0;
+    const int row = node / a.nx, x = node - row * a.nx, z = row / a.ny, y = row - z * a.ny;
+    const Nb b = make_nb(a, x, y, z);
+    if (own) {
+#define LBPC_CLA(q, ex, ey, ez, op)                                                      \
+        {                                                                               \
+            const bool w = b.template wall<ex, ey, ez>();                               \
+            const int m = w ? node : node + b.template off<ex, ey, ez>();               \
+            const int cta = m / per, at = m - cta * per;                                \
+            const unsigned base = shared_at(sm, (unsigned)cta);                         \
+            if constexpr (FLOW)                                                         \
+                af[q] = base + ((unsigned)(w ? op : q) * per + at) * (unsigned)sizeof(TFt); \
+            if constexpr (q >= 1 && q < 7) {                                            \
+                ag[q] = base + gbase +                                                  \
+                        ((unsigned)((w ? op : q) - 1) * per + at) * (unsigned)sizeof(TGt); \
+                const bool back = w && a.wall_iso[q - 1];                               \
+                if constexpr (sizeof(C) == 8)                                           \
+                    src[q] = back ? a.Tw[q - 1][face_index(a, q - 1, x, y, z)] : C(0);  \
+                else src[q] = back ? abb_source(a, k, q - 1, x, y, z) : C(0);           \
+                iso |= back ? 1u << q : 0u;                                             \
+            }                                                                           \
+        }
+        LBPC_Q19(LBPC_CLA)
+#undef LBPC_CLA
+        ep = hp[node];
+        if constexpr (!AA) {
+            if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT_PULL, false>(a, b, node, fs, f);
+            gather_g<Mode<P>::G, LAYOUT_PULL, false>(a, b, node, x, y, z, gs, g);
+        } else if (odd) {
+            if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT_AA_SWAPPED, false>(a, b, node, fs, f);
+            gather_g<Mode<P>::G, LAYOUT_AA_SWAPPED, false>(a, b, node, x, y, z, gs, g);
+        } else {
+            if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT_AA_NATURAL, false>(a, b, node, fs, f);
+            gather_g<Mode<P>::G, LAYOUT_AA_NATURAL, false>(a, b, node, x, y, z, gs, g);
+        }
+    }
+    double e = 0.0;
+    for (int i = 0;; i++) {
+        if (own) {
+            e = excess_plus<Mode<P>::G>(ep, g);
+            C T, fl;
+            invert_excess(a, e, T, fl);
+            C ux = C(0), uy = C(0), uz = C(0), rho, jx, jy, jz;
+            if constexpr (FLOW)
+                collide_flow<kRebuild<P>>(f, k, T, fl, ux, uy, uz, rho, jx, jy, jz);
+            collide_enth<C, !FLOW>(g, k, T, fl, ux, uy, uz);
+        }
+        if (i == n - 1) break;
+        const unsigned half = (unsigned)(i & 1);
+        if (own) {
+            TFt* bf = reinterpret_cast<TFt*>(sm + half * fhalf) + l;
+            TGt* bg = reinterpret_cast<TGt*>(sm + gbase + half * ghalf) + l;
+            if constexpr (FLOW)
+#pragma unroll
+                for (int q = 0; q < 19; q++) bf[q * per] = SF::enc(f[q], fshift(k, q));
+#pragma unroll
+            for (int q = 1; q < 7; q++) {
+                const TGt v = SG::enc_g(g[q], k.gshift);
+                bg[(q - 1) * per] = v;
+                g[q] = SG::dec(v, k.gshift);
+            }
+            ep = excess_minus<Mode<P>::G>(e, g);
+        }
+        cluster_barrier();
+        if (own) {
+            if constexpr (FLOW)
+#pragma unroll
+                for (int q = 0; q < 19; q++)
+                    f[q] = SF::dec(ld_cluster<TFt>(af[q] + half * fhalf), fshift(k, q));
+            // AA's odd step stores what comes back from a wall, in the storage precision
+            const bool stored = AA && ((odd + i) & 1);
+#pragma unroll
+            for (int q = 1; q < 7; q++) {
+                const C v = SG::dec(ld_cluster<TGt>(ag[q] + half * ghalf), k.gshift);
+                C r;  // abb_back
+                if constexpr (sizeof(C) == 8) r = std::fma(k.wT_cref, src[q], -v);
+                else r = -v + src[q];
+                g[q] = !(iso >> q & 1u) ? v
+                       : stored ? SG::dec(SG::enc_g(r, k.gshift), k.gshift) : SG::grid(r);
+            }
+        }
+    }
+    if (own) {
+        if constexpr (!AA) {
+            if constexpr (FLOW) scatter_f<Mode<P>::F, STEP_PULL>(a, b, node, fd, f);
+            scatter_g<Mode<P>::G, STEP_PULL>(a, b, node, x, y, z, gd, g);
+        } else if ((odd + n - 1) & 1) {
+            if constexpr (FLOW) scatter_f<Mode<P>::F, STEP_AA_ODD>(a, b, node, fd, f);
+            scatter_g<Mode<P>::G, STEP_AA_ODD>(a, b, node, x, y, z, gd, g);
+        } else {
+            if constexpr (FLOW) scatter_f<Mode<P>::F, STEP_AA_EVEN>(a, b, node, fd, f);
+            scatter_g<Mode<P>::G, STEP_AA_EVEN>(a, b, node, x, y, z, gd, g);
+        }
+        hp[node] = excess_minus<Mode<P>::G>(e, g);
+    }
+    cluster_barrier();  // no CTA leaves while another may still read its shared memory
+}
+
 template <class T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -2068,6 +2238,66 @@ struct Impl {
         }
     }
 
+    // Blocks of steps on one cluster.  Not with 16-bit f or the drag closure: a block of steps has to give the bits of the same
+    // steps one by one, and there the compiler fuses some products of the flow collision
+    // otherwise in the loop (a last-bit difference in FP32, which 16-bit storage amplifies).
+    static constexpr bool cluster_flow(int flow) {
+        return flow == 0 || (flow == 1 && !kRebuild<P>);
+    }
+    template <bool FLOW, bool AA>
+    static cudaError_t cluster_k(const Args& a, const void* fs, void* fd, const void* gs, void* gd,
+                                 double* hp, int n, int odd, int* fits, cudaStream_t s) {
+        auto* kern = k_steps_cluster<P, FLOW, AA>;
+        const int per = (a.N + CL_CTAS - 1) / CL_CTAS;
+        const size_t bytes = 2 * (size_t)per * ((FLOW ? 19 * sizeof(T) : 0) + 6 * sizeof(TGp));
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CL_CTAS;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t c{};
+        c.gridDim = dim3(CL_CTAS);
+        c.blockDim = dim3((per + 31) / 32 * 32);
+        c.dynamicSmemBytes = bytes;
+        c.stream = s;
+        c.attrs = at;
+        c.numAttrs = fits ? 1 : 2;
+        if (fits) return cudaOccupancyMaxActiveClusters(fits, kern, &c);
+        return cudaLaunchKernelEx(&c, kern, a, (const T*)fs, (T*)fd, (const TGp*)gs, (TGp*)gd, hp, n,
+                                  odd, per);
+    }
+    static cudaError_t cluster_f(const Args& a, bool aa, const void* fs, void* fd, const void* gs,
+                                 void* gd, double* hp, int n, int odd, int* fits, cudaStream_t s) {
+        if constexpr (cluster_flow(1))
+            if (a.flow)
+                return aa ? cluster_k<true, true>(a, fs, fd, gs, gd, hp, n, odd, fits, s)
+                          : cluster_k<true, false>(a, fs, fd, gs, gd, hp, n, odd, fits, s);
+        return aa ? cluster_k<false, true>(a, fs, fd, gs, gd, hp, n, odd, fits, s)
+                  : cluster_k<false, false>(a, fs, fd, gs, gd, hp, n, odd, fits, s);
+    }
+    static bool cluster_fits(const Args& a, bool aa) {
+        const int flow = a.flow ? (coef<CT<P>>(a).darcy ? 2 : 1) : 0;
+        if (!cluster_flow(flow)) return false;
+        if (a.N > CL_CTAS * (flow ? CL_THREADS<P, true> : CL_THREADS<P, false>)) return false;
+        int fits = 0;
+        if (cluster_f(a, aa, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0, &fits, nullptr) !=
+            cudaSuccess) {
+            cudaGetLastError();  // no such cluster on this device: the step-by-step path
+            return false;
+        }
+        return fits > 0;
+    }
+    static cudaError_t cluster_steps(const Args& a, bool aa, const void* fs, void* fd,
+                                     const void* gs, void* gd, double* hp, int n, int odd,
+                                     cudaStream_t s) {
+        return cluster_f(a, aa, fs, fd, gs, gd, hp, n, odd, nullptr, s);
+    }
+
     template <int LAYOUT, bool FLOW>
     static void macro_k(const Args& a, const void* f, const void* g, const double* hp,
                         const MacroOut& o, cudaStream_t s) {
@@ -2154,7 +2384,7 @@ struct Impl {
     }
 
     static const Launchers& table() {
-        static const Launchers L = {&step, &macro, &init, &dist, &step_tape, &adj_seed,
+        static const Launchers L = {&step, &cluster_fits, &cluster_steps, &macro, &init, &dist, &step_tape, &adj_seed,
                                     &adj_reverse, &check, sizeof(T), sizeof(TGp),
                                     sizeof(CT<P>)};
         return L;
