@@ -71,18 +71,27 @@ WsLayout ws_layout(int nx, int ny, int nz, const lbpc_params* p) {
     return w;
 }
 
-// Fixed-order sum of n partials into out[0] (one block).
-__global__ void __launch_bounds__(256) k_sum(const double* __restrict__ p, int n, double* out) {
-    __shared__ double sh[256];
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) acc += p[i];
-    sh[threadIdx.x] = acc;
+// Fixed-order sums of n partials: block b sums its share of consecutive values into out[b].
+// Four loads in flight per thread: one block waiting for one load after another took 68 us on
+// the 27,648 warp partials of 96^3.
+constexpr int SUM_THREADS = 256;
+__global__ void __launch_bounds__(SUM_THREADS) k_sum(const double* __restrict__ p, int n, double* out) {
+    __shared__ double sh[SUM_THREADS];
+    const long long share = ((long long)n + gridDim.x - 1) / gridDim.x;
+    const long long lo = blockIdx.x * share, hi = lo + share < n ? lo + share : n;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (long long i = lo + threadIdx.x; i < hi; i += 4 * SUM_THREADS) {
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (i + k * SUM_THREADS < hi) acc[k] += p[i + k * SUM_THREADS];
+    }
+    sh[threadIdx.x] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     __syncthreads();
-    for (int st = 128; st > 0; st >>= 1) {
+    for (int st = SUM_THREADS / 2; st > 0; st >>= 1) {
         if ((int)threadIdx.x < st) sh[threadIdx.x] += sh[threadIdx.x + st];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = sh[0];
+    if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
 }
 
 __global__ void k_fill(double* p, double v, int n) {
@@ -109,17 +118,25 @@ k_finalize(const double* __restrict__ partial, const double* __restrict__ lines,
             for (int k = 0; k < NRED; k++) sh[threadIdx.x][k] += sh[threadIdx.x + s][k];
         __syncthreads();
     }
+    // first node of each front line with f_l < 1/2 (nx: none), by all threads: one thread
+    // walking the lines took 30 us of a diagnostics point at nx = 160
+    __shared__ int first[3];
+    if (threadIdx.x < 3) first[threadIdx.x] = nx;
+    __syncthreads();
+    for (int l = 0; l < 3; l++) {
+        int m = nx;
+        for (int x = threadIdx.x; x < nx && m == nx; x += blockDim.x)
+            if (lines[(size_t)l * nx + x] < 0.5) m = x;
+        if (m < nx) atomicMin(&first[l], m);
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
     double front = 0.0;
     for (int l = 0; l < 3; l++) {
         const double* v = lines + (size_t)l * nx;
+        const int x = first[l];
         double xc = nx;  // no crossing: the whole line is liquid
-        for (int x = 0; x < nx; x++) {
-            if (v[x] < 0.5) {
-                xc = x == 0 ? -0.5 : (x - 1) + (v[x - 1] - 0.5) / (v[x - 1] - v[x]);
-                break;
-            }
-        }
+        if (x < nx) xc = x == 0 ? -0.5 : (x - 1) + (v[x - 1] - 0.5) / (v[x - 1] - v[x]);
         front += (xc + 0.5) / 3.0;
     }
     double r[LBPC_S_COUNT];
@@ -244,7 +261,7 @@ lbpc_status init_state(lbpc_handle* h, const double* Qf, const double* Qg, const
     void* g = h->p.streaming == LBPC_PULL ? h->g[h->cur] : h->g[0];
     const Layout lay = h->p.streaming == LBPC_PULL ? LAYOUT_PULL : LAYOUT_AA_NATURAL;
     h->L->init(h->args, lay, Qf, Qg, h0, f, g, h->hp, h->stream);
-    h->launches += 2;
+    h->launches++;
     LBPC_CK(h, cudaGetLastError());
     return LBPC_OK;
 }
@@ -796,8 +813,9 @@ lbpc_status lbpc_adjoint_forward(lbpc_handle* h, int nsteps, int ckpt_every, voi
         h->launches++;
     }
     // seed lambda_N = d f_l / dh (and J = sum f_l, the direct dJ/dL part)
-    h->L->adj_seed(h->args, h->g[h->cur], h->hp, A.lam[0], A.Lpart, A.Jpart, h->stream);
-    k_sum<<<1, 256, 0, h->stream>>>(A.Jpart, A.nblocks, A.red);
+    LBPC_CK(h, cudaMemsetAsync(A.Lpart, 0, sizeof(double) * A.nwarps, h->stream));
+    const int nj = h->L->adj_seed(h->args, h->g[h->cur], h->hp, A.lam[0], A.Lpart, A.Jpart, h->stream);
+    k_sum<<<1, SUM_THREADS, 0, h->stream>>>(A.Jpart, nj, A.red);
     h->launches += 2;
     LBPC_CK(h, cudaGetLastError());
     double J = 0.0;
@@ -848,8 +866,11 @@ lbpc_status lbpc_adjoint_backward(lbpc_handle* h, int face, double* dJ_dTw_host,
         }
         h->launches += len;
     }
-    k_sum<<<1, 256, 0, h->stream>>>(A.Lpart, A.nwarps, A.red + 1);
-    h->launches++;
+    // in two stages over the J partials' space, which is free by now
+    const int nl = std::min(A.nblocks, (A.nwarps + 1023) / 1024);
+    k_sum<<<nl, SUM_THREADS, 0, h->stream>>>(A.Lpart, A.nwarps, A.Jpart);
+    k_sum<<<1, SUM_THREADS, 0, h->stream>>>(A.Jpart, nl, A.red + 1);
+    h->launches += 2;
     LBPC_CK(h, cudaGetLastError());
     double dJdL = 0.0;
     LBPC_CK(h, cudaMemcpyAsync(&dJdL, A.red + 1, sizeof(double), cudaMemcpyDeviceToHost, h->stream));

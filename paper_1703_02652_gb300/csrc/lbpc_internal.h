@@ -119,8 +119,8 @@ struct Launchers {
     // 4N compute-precision values), seed of lambda at the final state, one reverse step
     void (*step_tape)(const Args&, const void* fs, void* fd, const void* gs, void* gd,
                       double* hp, void* tape_e, void* tape_m, cudaStream_t);
-    void (*adj_seed)(const Args&, const void* gs, const double* hp, void* lam, double* Lpart,
-                     double* Jpart, cudaStream_t);
+    int (*adj_seed)(const Args&, const void* gs, const double* hp, void* lam, double* Lpart,
+                    double* Jpart, cudaStream_t);  // number of J partials
     void (*adj_reverse)(const Args&, const void* lin, void* lout, const void* tape_e,
                         const void* tape_m, int wface, double* gtw, double* Lpart, cudaStream_t);
     // divergence check: *flag = 1 if a stored g population or h' is not finite (the flag

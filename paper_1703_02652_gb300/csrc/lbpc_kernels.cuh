@@ -12,6 +12,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -118,6 +119,66 @@ LBPC_HD float d2f_near(double v) {
 #else
     if (std::fabs(v) < 1.1754943508222875e-38) return std::signbit(v) ? -0.0f : 0.0f;
     return (float)v;
+#endif
+}
+
+// Conversions for the read-out and set-up kernels, as the hardware's (every value, infinities
+// and NaN included) but by integer operations: those instructions run on the FP64 pipe, whose
+// two lanes per SM bounded these kernels (25 conversions per node; a warp's takes 16 cycles).
+LBPC_HD double f2d(float v) {
+#if defined(__CUDA_ARCH__)
+    const bool small = (__float_as_uint(v) & 0x7f800000u) == 0;  // zero or subnormal
+    const unsigned u = __float_as_uint(small ? v * 0x1p64f : v);
+    const unsigned mag = u & 0x7fffffffu;
+    unsigned bias = small ? 896u - 64u : 896u;
+    if (mag >= 0x7f800000u) bias = 2u * 896u;
+    const unsigned long long bits = ((unsigned long long)mag << 29) +
+                                    (mag ? (unsigned long long)bias << 52 : 0ull);
+    return __longlong_as_double((long long)(bits | ((unsigned long long)(u >> 31) << 63)));
+#else
+    return (double)v;
+#endif
+}
+LBPC_HD double f2d(double v) { return v; }
+// The bits of a double by halves: the compiler turns some tests on the whole 64-bit pattern
+// back into comparisons on the FP64 pipe.
+#if defined(__CUDA_ARCH__)
+__device__ __forceinline__ unsigned long long bits_of(double v) {
+    return (unsigned long long)(unsigned)__double2hiint(v) << 32 | (unsigned)__double2loint(v);
+}
+#endif
+// double -> compute precision, round to nearest even.  Anything but zero and normal floats sets
+// `rare` and has to be converted by the hardware (HW).
+template <class C, bool HW> LBPC_HD C d2c(double v, bool& rare) {
+#if defined(__CUDA_ARCH__)
+    if constexpr (sizeof(C) == 4 && !HW) {
+        const unsigned long long u = bits_of(v);
+        const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+        unsigned long long m = u & 0x7fffffffffffffffull;
+        const bool zero = m == 0;
+        m += 0x0fffffffull + ((m >> 29) & 1ull);
+        // a normal float lies between 2^-126 (exponent 897 here) and 2^128 (1151)
+        rare |= !zero && (m < (897ull << 52) || m >= (1151ull << 52));
+        const unsigned r = (unsigned)((m >> 29) - (896ull << 23));
+        return __uint_as_float(sign | (zero ? 0u : r));
+    }
+#endif
+    (void)rare;
+    return (C)v;
+}
+// Not finite, by the exponent bits.
+LBPC_HD bool not_finite(double v) {
+#if defined(__CUDA_ARCH__)
+    return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000;
+#else
+    return !std::isfinite(v);
+#endif
+}
+LBPC_HD bool not_finite(float v) {
+#if defined(__CUDA_ARCH__)
+    return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u;
+#else
+    return !std::isfinite(v);
 #endif
 }
 
@@ -433,18 +494,26 @@ LBPC_HD void scatter_g(const Args& a, const NB& b, int n, int x, int y, int z,
 // an ulp of 0 or L, where both branches give the same T and f_l to that accuracy.  (Exact
 // branch tests on the bits of e measured 2% slower on the 16-bit step, an FP64 fused
 // multiply-add for the value 5%.)
+//
+// The FP64 branch is found from the bits (a comparison is an operation of the FP64 pipe) and
+// its values take three FP64 operations in all.  NaN is neither solid nor liquid.
+struct Phase { bool solid, liquid; };
+LBPC_HD Phase phase_of(double e, double L) {
+#if defined(__CUDA_ARCH__)
+    const long long u = (long long)bits_of(e), m = u & 0x7fffffffffffffffll;
+    const bool number = m <= 0x7ff0000000000000ll;
+    return {number && (u < 0 || m == 0), number && u >= (long long)bits_of(L)};  // L > 0
+#else
+    return {e <= 0.0, e >= L};
+#endif
+}
 LBPC_HD void invert_excess(const Args& a, double e, double& T, double& fl) {
     const Coef<double>& k = a.cd;
-    if (e <= 0.0) {
-        fl = 0.0;
-        T = k.Tm + e * k.Cps_inv;
-    } else if (e >= k.L) {
-        fl = 1.0;
-        T = k.Tm + (e - k.L) * k.Cpl_inv;
-    } else {
-        fl = e * k.L_inv;
-        T = k.Tm;
-    }
+    const Phase ph = phase_of(e, k.L);
+    const double d = ph.liquid ? e - k.L : e;
+    const double t = k.Tm + d * (ph.liquid ? k.Cpl_inv : k.Cps_inv);
+    T = ph.solid || ph.liquid ? t : k.Tm;
+    fl = ph.liquid ? 1.0 : (ph.solid ? 0.0 : e * k.L_inv);
 }
 LBPC_HD void invert_excess(const Args& a, double e, float& T, float& fl) {
     const Coef<float>& k = a.cf;
@@ -1134,133 +1203,173 @@ LBPC_HD void step_pair_aa(const Args& a, int x0, int y, int z, TF<P>* F, TG<P>* 
         make_double2(excess_minus<Mode<P>::G>(e0, g0), excess_minus<Mode<P>::G>(e1, g1));
 }
 
-// Macroscopic state of node n and its contributions to the diagnostics sums
-// (acc: sum f_l, sum h, sum rho, -x wall flux, -x wall gradient, non-finite count).
-template <int P, int LAYOUT, bool FLOW>
-LBPC_HD void macro_node(const Args& a, int n, const TF<P>* fs,
-                        const TG<P>* gs, const double* hp, const MacroOut& out,
-                        double* acc) {
+// Diagnostics sums of one thread.  Few FP64 operations per node: the liquid nodes are counted,
+// only mushy ones add a fraction, and h_s enters once per thread.
+struct MacroSums {
+    double fl, e, rho, flux, grad;  // mushy f_l; h - h_s; rho; -x wall flux and gradient
+    int liquid, bad, nodes;         // liquid, non-finite and all nodes
+};
+#if defined(__CUDACC__)
+// (out of line, so that the warps without a mushy node skip the FP64 operations)
+__device__ __noinline__ inline void add_mushy(double& fl, double e, double L_inv) { fl += e * L_inv; }
+#endif
+
+// Macroscopic state of node (x, y, z): with SUMS its contributions to the diagnostics sums and
+// the front lines, otherwise its fields.
+template <int P, int LAYOUT, bool FLOW, bool SUMS>
+LBPC_HD void macro_node(const Args& a, int x, int y, int z, const TF<P>* fs, const TG<P>* gs,
+                        const double* hp, const MacroOut& out, MacroSums& acc) {
     using C = CT<P>;
     const Coef<C>& k = coef<C>(a);
-    const int x = n % a.nx, y = (n / a.nx) % a.ny, z = n / (a.nx * a.ny);
-    const Nb b = make_nb(a, x, y, z);
+    const int n = x + a.nx * (y + a.ny * z);
     C f[19], g[7];
-    if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
-    gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
+    if (is_interior(a, x, y, z)) {
+        const NbInterior b{a.nx, a.nx * a.ny};
+        if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
+        gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
+    } else {
+        const Nb b = make_nb(a, x, y, z);
+        if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
+        gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
+    }
     const double e = excess_plus<Mode<P>::G>(hp[n], g);
-    const double h = a.hs + e;
-    double Td, fld;  // reported: the FP64 inversion
-    invert_excess(a, e, Td, fld);
     C rho = C(0), ux = C(0), uy = C(0), uz = C(0);
     if constexpr (FLOW) {  // the velocity as the step computes it
         C T, fl, jx, jy, jz, Fx, Fy, Fz;
         invert_excess(a, e, T, fl);
         flow_macro(f, k, T, fl, rho, jx, jy, jz, ux, uy, uz, Fx, Fy, Fz);
     }
-    if (out.T) out.T[n] = Td;
-    if (out.fl) out.fl[n] = fld;
-    if (out.h) out.h[n] = h;
-    if (out.rho) out.rho[n] = (double)rho;
-    if (out.ux) out.ux[n] = (double)ux;
-    if (out.uy) out.uy[n] = (double)uy;
-    if (out.uz) out.uz[n] = (double)uz;
-    if (acc) {
-        acc[0] += fld;
-        acc[1] += h;
-        acc[2] += (double)rho;
-        if (x == 0) {
-            const double Tw = a.Tw[0][y + a.ny * z];
-            if (a.wall_iso[0]) acc[3] += 2.0 * ((double)g[1] + (double)k.gshift) - (double)k.wT_cref * Tw;
-            acc[4] += (Tw - Td) * 2.0;
+    if constexpr (!SUMS) {
+        double Td, fld;  // the FP64 inversion
+        invert_excess(a, e, Td, fld);
+        if (out.T) out.T[n] = Td;
+        if (out.fl) out.fl[n] = fld;
+        if (out.h) out.h[n] = a.hs + e;
+        if (out.rho) out.rho[n] = f2d(rho);
+        if (out.ux) out.ux[n] = f2d(ux);
+        if (out.uy) out.uy[n] = f2d(uy);
+        if (out.uz) out.uz[n] = f2d(uz);
+    } else {
+#if defined(__CUDACC__)
+        const Phase ph = phase_of(e, a.cd.L);
+        if (ph.liquid) acc.liquid++;
+        else if (!ph.solid) add_mushy(acc.fl, e, a.cd.L_inv);
+        acc.nodes++;
+        acc.e += e;
+        if constexpr (FLOW) acc.rho += f2d(rho);
+        if (x == 0 || y == a.ny / 2) {
+            double Td, fld;
+            invert_excess(a, e, Td, fld);
+            if (x == 0) {
+                const double Tw = a.Tw[0][y + a.ny * z];
+                if (a.wall_iso[0])
+                    acc.flux += 2.0 * (f2d(g[1]) + f2d(k.gshift)) - f2d(k.wT_cref) * Tw;
+                acc.grad += (Tw - Td) * 2.0;
+            }
+            if (y == a.ny / 2) {
+                if (z == a.nz / 4) out.lines[x] = fld;
+                if (z == a.nz / 2) out.lines[a.nx + x] = fld;
+                if (z == (3 * a.nz) / 4) out.lines[2 * a.nx + x] = fld;
+            }
         }
         const C gsum = ((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]);
-        if (!isfinite(h) || !isfinite((double)rho) || !isfinite((double)gsum)) acc[5] += 1.0;
-    }
-    if (out.lines && y == a.ny / 2) {
-        if (z == a.nz / 4) out.lines[x] = fld;
-        if (z == a.nz / 2) out.lines[a.nx + x] = fld;
-        if (z == (3 * a.nz) / 4) out.lines[2 * a.nx + x] = fld;
+        if (not_finite(e) || not_finite(rho) || not_finite(gsum)) acc.bad++;
+#endif
     }
 }
 
-// Value of pre-collision population q of node m in the state to load: Q when given,
-// else the rest equilibrium of f (rho = 1, u = 0) and g^eq(h0, T(h0), 0) of Eq. 7.
-template <class C>
-LBPC_HD double state_f(const double* Qf, size_t N, int q, int m) {
-    return Qf ? Qf[(size_t)q * N + m] : (q == 0 ? 1.0 / 3.0 : (q < 7 ? 1.0 / 18.0 : 1.0 / 36.0));
-}
-template <class C>
-LBPC_HD double state_g(const Args& a, const Coef<C>& k, const double* Qg, const double* h0,
-                       int q, int m) {
-    if (Qg) return Qg[(size_t)q * a.N + m];
-    C T, fl;
-    invert_excess(a, h0[m] - a.hs, T, fl);
-    return (double)(k.wa_cref * T);
-}
-
-// Write the slots of node (x, y, z) so that a gather in LAYOUT returns the state Q.
-// For the pull layout a slot holds the value its downwind neighbour pulls; slots whose
-// downwind neighbour lies behind a wall feed the node's own bounce-back.
-template <int P, int LAYOUT, bool FLOW>
-LBPC_HD void init_node(const Args& a, int x, int y, int z, const double* Qf, const double* Qg,
-                       const double* h0, TF<P>* fd, TG<P>* gd) {
+// Load the pre-collision state of node (x, y, z) so that a gather in LAYOUT returns it: the
+// node's values go where its gather reads them (pull: the upwind node's slot, or at a wall
+// the reflected slot of the node itself, with the inverse wall rule), and the rest channel e' =
+// h - h_s - sum_a g_a takes the g values as that gather will return them, in the storage
+// precision.  The state is Q when given, else the rest equilibrium of f (rho = 1, u = 0) and
+// g^eq(h0, T(h0), 0) of Eq. 7.  One pass in which a node reads its own values only: pulling
+// each slot's value from the downwind node took seven inversions per node and a second pass for
+// e' (128^3 BF16 from arrays: 292 us, from h0 at 96^3 FP32: 136 us; see k_init).
+// Returns whether a value needs the hardware's conversion (HW).
+template <int P, int LAYOUT, bool FLOW, bool HW>
+LBPC_HD bool init_node(const Args& a, int x, int y, int z, const double* Qf, const double* Qg,
+                       const double* h0, TF<P>* fd, TG<P>* gd, double* hp) {
     using C = CT<P>;
+    using SF = Store<Mode<P>::F>;
+    using SG = Store<Mode<P>::G>;
     const Coef<C>& k = coef<C>(a);
     const int n = x + a.nx * (y + a.ny * z);
-    const Nb b = make_nb(a, x, y, z);
     const size_t N = (size_t)a.N;
+    const Nb b = make_nb(a, x, y, z);
+    bool rare = false;
     if constexpr (FLOW) {
+        const double sh[3] = {f2d(k.fshift0), f2d(k.fshift1), f2d(k.fshift2)};
+        C c[19];
+        if (Qf) {
+            double v[19];
+#pragma unroll
+            for (int q = 0; q < 19; q++) v[q] = Qf[(size_t)q * N + n];
+#pragma unroll
+            for (int q = 0; q < 19; q++) {
+                if constexpr (sizeof(C) == 4) v[q] -= sh[q == 0 ? 0 : (q < 7 ? 1 : 2)];
+                c[q] = d2c<C, HW>(v[q], rare);
+            }
+        } else {
+            const double w[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0};
+            C r[3];
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+                r[i] = d2c<C, HW>(sizeof(C) == 4 ? w[i] - sh[i] : w[i], rare);
+#pragma unroll
+            for (int q = 0; q < 19; q++) c[q] = r[q == 0 ? 0 : (q < 7 ? 1 : 2)];
+        }
 #define LBPC_IF(q, ex, ey, ez, op)                                                       \
         {                                                                               \
-            double v;                                                                   \
-            if constexpr (LAYOUT == LAYOUT_AA_NATURAL) v = state_f<C>(Qf, N, q, n);     \
-            else {                                                                      \
-                const bool w = b.template wall<-(ex), -(ey), -(ez)>();                         \
-                v = w ? state_f<C>(Qf, N, op, n)                                        \
-                      : state_f<C>(Qf, N, q, n + b.template off<-(ex), -(ey), -(ez)>());       \
-            }                                                                           \
-            fd[(size_t)q * N + n] = Store<Mode<P>::F>::enc((C)(v - (double)fshift(k, q)), C(0)); \
+            const bool w = LAYOUT == LAYOUT_PULL && b.template wall<ex, ey, ez>();      \
+            const int off = LAYOUT == LAYOUT_PULL ? b.template off<ex, ey, ez>() : 0;   \
+            fd[(size_t)(w ? op : q) * N + (w ? n : n + off)] = SF::enc(c[q], C(0));     \
         }
         LBPC_Q19(LBPC_IF)
 #undef LBPC_IF
     }
+    double h, v[7];
+    if (Qg) {
+#pragma unroll
+        for (int q = 0; q < 7; q++) v[q] = Qg[(size_t)q * N + n];
+        h = v[0];
+#pragma unroll
+        for (int q = 1; q < 7; q++) h += v[q];
+    } else {
+        h = h0[n];
+        C T, fl;
+        invert_excess(a, h - a.hs, T, fl);
+#pragma unroll
+        for (int q = 1; q < 7; q++) v[q] = f2d(k.wa_cref * T);
+    }
+    C g[7];
+    typename SG::T t[7];
+#pragma unroll
+    for (int q = 1; q < 7; q++) {
+        t[q] = SG::enc_g(d2c<C, HW>(SG::kGrid ? v[q] - f2d(k.gshift) : v[q], rare), C(0));
+        g[q] = SG::dec(t[q], k.gshift);
+    }
+    if constexpr (LAYOUT == LAYOUT_PULL) {
+#define LBPC_IW(q, ex, ey, ez, op)                                                       \
+        if (b.template wall<ex, ey, ez>() && a.wall_iso[q - 1]) {                        \
+            double d = f2d(k.wT_cref) * a.Tw[q - 1][face_index(a, q - 1, x, y, z)] - v[q]; \
+            if constexpr (SG::kGrid) d -= f2d(k.gshift);                                \
+            t[q] = SG::enc_g(d2c<C, HW>(d, rare), C(0));                                \
+            g[q] = SG::grid(abb_back(a, k, q - 1, x, y, z, SG::dec(t[q], k.gshift)));   \
+        }
+        LBPC_Q7(LBPC_IW)
+#undef LBPC_IW
+    }
 #define LBPC_IG(q, ex, ey, ez, op)                                                       \
     {                                                                                   \
-        double v;                                                                       \
-        if constexpr (LAYOUT == LAYOUT_AA_NATURAL) v = state_g(a, k, Qg, h0, q, n);     \
-        else {                                                                          \
-            const bool w = b.template wall<-(ex), -(ey), -(ez)>();                             \
-            if (w) {                                                                    \
-                v = state_g(a, k, Qg, h0, op, n);                                       \
-                if (a.wall_iso[op - 1])                                                 \
-                    v = (double)k.wT_cref * a.Tw[op - 1][face_index(a, op - 1, x, y, z)] - v; \
-            } else {                                                                    \
-                v = state_g(a, k, Qg, h0, q, n + b.template off<-(ex), -(ey), -(ez)>());       \
-            }                                                                           \
-        }                                                                               \
-        gd[(size_t)(q - 1) * N + n] = Store<Mode<P>::G>::enc_g((C)(v - (double)k.gshift), C(0)); \
+        const bool w = LAYOUT == LAYOUT_PULL && b.template wall<ex, ey, ez>();          \
+        const int off = LAYOUT == LAYOUT_PULL ? b.template off<ex, ey, ez>() : 0;       \
+        gd[(size_t)((w ? op : q) - 1) * N + (w ? n : n + off)] = t[q];                  \
     }
     LBPC_Q7(LBPC_IG)
 #undef LBPC_IG
-}
-
-// e' = h - h_s - sum_a g_a(gathered), so that the stored state reproduces h.
-template <int P, int LAYOUT>
-LBPC_HD void init_hprime_node(const Args& a, int x, int y, int z, const double* Qg,
-                              const double* h0, const TG<P>* gs, double* hp) {
-    using C = CT<P>;
-    const int n = x + a.nx * (y + a.ny * z);
-    const Nb b = make_nb(a, x, y, z);
-    double h;
-    if (Qg) {
-        h = 0.0;
-        for (int q = 0; q < 7; q++) h += Qg[(size_t)q * a.N + n];
-    } else {
-        h = h0[n];
-    }
-    C g[7];
-    gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
     hp[n] = excess_minus<Mode<P>::G>(h - a.hs, g);
+    return rare;
 }
 
 // Pre-collision populations of node (x, y, z) in FP64 (g_0 = h' = h_s + e').
@@ -1269,20 +1378,28 @@ LBPC_HD void dist_node(const Args& a, int x, int y, int z, const TF<P>* fs,
                        const TG<P>* gs, const double* hp, double* Qf, double* Qg) {
     using C = CT<P>;
     const int n = x + a.nx * (y + a.ny * z);
-    const Nb b = make_nb(a, x, y, z);
     const size_t N = (size_t)a.N;
     const Coef<C>& k = coef<C>(a);
-    C g[7];
-    gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
-    const double gs_ = (double)k.gshift;
+    const bool with_f = FLOW && Qf;
+    C f[19], g[7];
+    if (is_interior(a, x, y, z)) {
+        const NbInterior b{a.nx, a.nx * a.ny};
+        if (with_f) gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
+        gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
+    } else {
+        const Nb b = make_nb(a, x, y, z);
+        if (with_f) gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
+        gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
+    }
+    const double gs_ = f2d(k.gshift);
     Qg[n] = a.hs + hp[n] - 6.0 * gs_;
-    for (int q = 1; q < 7; q++) Qg[(size_t)q * N + n] = (double)g[q] + gs_;
-    if constexpr (FLOW) {
-        if (Qf) {
-            C f[19];
-            gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
-            for (int q = 0; q < 19; q++) Qf[(size_t)q * N + n] = (double)f[q] + (double)fshift(k, q);
-        }
+    for (int q = 1; q < 7; q++)
+        Qg[(size_t)q * N + n] = Store<Mode<P>::G>::kGrid ? f2d(g[q]) + gs_ : f2d(g[q]);
+    if (with_f) {
+        const double sh[3] = {f2d(k.fshift0), f2d(k.fshift1), f2d(k.fshift2)};
+        for (int q = 0; q < 19; q++)
+            Qf[(size_t)q * N + n] =
+                sizeof(C) == 8 ? (double)f[q] : f2d(f[q]) + sh[q == 0 ? 0 : (q < 7 ? 1 : 2)];
     }
 }
 
@@ -1511,9 +1628,11 @@ LBPC_HD CT<P> adj_seed_node(const Args& a, int x, int y, int z,
     using C = CT<P>;
     const Coef<C>& k = coef<C>(a);
     const int n = x + a.nx * (y + a.ny * z);
-    const Nb b = make_nb(a, x, y, z);
     C g[7];
-    gather_g<Mode<P>::G, LAYOUT_PULL, true>(a, b, n, x, y, z, gs, g);
+    if (is_interior(a, x, y, z))
+        gather_g<Mode<P>::G, LAYOUT_PULL, true>(a, NbInterior{a.nx, a.nx * a.ny}, n, x, y, z, gs, g);
+    else
+        gather_g<Mode<P>::G, LAYOUT_PULL, true>(a, make_nb(a, x, y, z), n, x, y, z, gs, g);
     const double e = excess_plus<Mode<P>::G>(hp[n], g);
     C T, fl, dTde, dfde, dTdL, dfdL;
     invert_excess_d(k, tape_excess(a, e, C(0)), T, fl, dTde, dfde, dTdL, dfdL);
@@ -1521,7 +1640,7 @@ LBPC_HD CT<P> adj_seed_node(const Args& a, int x, int y, int z,
     const int nf = FLOW ? 19 : 0;
     for (int q = 0; q < nf; q++) lam[(size_t)q * N + n] = C(0);
     for (int q = 0; q < 7; q++) lam[(size_t)(nf + q) * N + n] = dfde;
-    fl_out = (double)fl;
+    fl_out = f2d(fl);
     return dfdL;
 }
 
@@ -1988,49 +2107,58 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
-// Macroscopic fields of the current state and FP64 block partial sums for diagnostics
-// (grid-stride over nodes; one partial row per block, summed later in a fixed order).
-template <int P, int LAYOUT, bool FLOW>
-__global__ void __launch_bounds__(RED_THREADS)
+// Macroscopic fields of the current state, or (SUMS) FP64 block partial sums for diagnostics:
+// grid-stride over nodes, one partial row per block, summed later in a fixed order.
+template <int P, int LAYOUT, bool FLOW, bool SUMS>
+__global__ void __launch_bounds__(RED_THREADS, P == LBPC_FP64 ? 2 : 3)
 k_macro(const __grid_constant__ Args a, const TF<P>* __restrict__ fs,
         const TG<P>* __restrict__ gs, const double* __restrict__ hp,
         const MacroOut out) {
-    double acc[NRED] = {0, 0, 0, 0, 0, 0};
+    if (SUMS && (long long)blockIdx.x * RED_THREADS >= a.N) {  // no node: a row of zeros
+        if (threadIdx.x < NRED) out.partial[blockIdx.x * NRED + threadIdx.x] = 0.0;
+        return;
+    }
+    MacroSums m{};
     // 64-bit loop index: n + stride may pass 2^31 - 1 near the node limit
     for (long long n = blockIdx.x * blockDim.x + threadIdx.x; n < a.N;
-         n += (long long)gridDim.x * blockDim.x)
-        macro_node<P, LAYOUT, FLOW>(a, (int)n, fs, gs, hp, out, out.partial ? acc : nullptr);
-    if (!out.partial) return;
-    __shared__ double sh[RED_THREADS / 32][NRED];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NRED; i++) {
-        const double v = warp_sum(acc[i]);
-        if (lane == 0) sh[wid][i] = v;
+         n += (long long)gridDim.x * blockDim.x) {
+        const int row = (int)a.by_nx.div((unsigned)n), x = (int)n - row * a.nx;
+        const int z = (int)a.by_ny.div((unsigned)row), y = row - z * a.ny;
+        macro_node<P, LAYOUT, FLOW, SUMS>(a, x, y, z, fs, gs, hp, out, m);
     }
-    __syncthreads();
-    if (threadIdx.x < NRED) {
-        double s = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; w++) s += sh[w][threadIdx.x];
-        out.partial[blockIdx.x * NRED + threadIdx.x] = s;
+    if constexpr (SUMS) {
+        // tree over the block in shared memory: a third of the FP64 operations of warp shuffles
+        const double acc[NRED] = {m.fl + m.liquid, m.nodes * a.hs + m.e, m.rho, m.flux, m.grad,
+                                  (double)m.bad};
+        __shared__ double sh[NRED][RED_THREADS];
+        const int t = threadIdx.x;
+#pragma unroll
+        for (int i = 0; i < NRED; i++) sh[i][t] = acc[i];
+        __syncthreads();
+        for (int st = RED_THREADS / 2; st > 0; st >>= 1) {
+            if (t < st)
+#pragma unroll
+                for (int i = 0; i < NRED; i++) sh[i][t] += sh[i][t + st];
+            __syncthreads();
+        }
+        if (t < NRED) out.partial[blockIdx.x * NRED + t] = sh[t][0];
     }
 }
 
 template <int P, int LAYOUT, bool FLOW>
+__device__ __noinline__ void init_node_hw(const Args& a, int x, int y, int z, const double* Qf,
+                                          const double* Qg, const double* h0, TF<P>* fd, TG<P>* gd,
+                                          double* hp) {
+    init_node<P, LAYOUT, FLOW, true>(a, x, y, z, Qf, Qg, h0, fd, gd, hp);
+}
+template <int P, int LAYOUT, bool FLOW>
 __global__ void __launch_bounds__(STEP_THREADS)
 k_init(const __grid_constant__ Args a, const double* __restrict__ Qf, const double* __restrict__ Qg,
-       const double* __restrict__ h0, TF<P>* fd, TG<P>* gd) {
+       const double* __restrict__ h0, TF<P>* fd, TG<P>* gd, double* hp) {
     LBPC_NODE_XYZ
-    init_node<P, LAYOUT, FLOW>(a, x, y, z, Qf, Qg, h0, fd, gd);
-}
-
-template <int P, int LAYOUT>
-__global__ void __launch_bounds__(STEP_THREADS)
-k_init_hprime(const __grid_constant__ Args a, const double* __restrict__ Qg,
-              const double* __restrict__ h0, const TG<P>* __restrict__ gs,
-              double* __restrict__ hp) {
-    LBPC_NODE_XYZ
-    init_hprime_node<P, LAYOUT>(a, x, y, z, Qg, h0, gs, hp);
+    // a node's slots are its own: writing them again is safe
+    if (init_node<P, LAYOUT, FLOW, false>(a, x, y, z, Qf, Qg, h0, fd, gd, hp))
+        init_node_hw<P, LAYOUT, FLOW>(a, x, y, z, Qf, Qg, h0, fd, gd, hp);
 }
 
 template <int P, int LAYOUT, bool FLOW>
@@ -2099,17 +2227,26 @@ __device__ __forceinline__ int warp_slot() {
     return block_linear() * (STEP_THREADS / 32) + (block_thread() >> 5);
 }
 
+// Grid-stride over the nodes, so that a node costs two FP64 additions instead of its share of
+// two FP64 warp reductions (96^3 FP32: 46 us, 26 of them on the FP64 pipe, with one node per
+// thread).  Lpart is zero before: only this grid's warps write their slots.
 template <int P, bool FLOW>
 __global__ void __launch_bounds__(STEP_THREADS)
 k_adj_seed(const __grid_constant__ Args a, const TG<P>* __restrict__ gs,
            const double* __restrict__ hp, CT<P>* __restrict__ lam,
            double* __restrict__ Lpart, double* __restrict__ Jpart) {
-    int x, y, z;
-    double dL = 0.0, fl = 0.0;
-    if (item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z)) dL = (double)adj_seed_node<P, FLOW>(a, x, y, z, gs, hp, lam, fl);
+    double dL = 0.0, J = 0.0;
+    for (long long n = blockIdx.x * blockDim.x + threadIdx.x; n < a.N;
+         n += (long long)gridDim.x * blockDim.x) {
+        const int row = (int)a.by_nx.div((unsigned)n), x = (int)n - row * a.nx;
+        const int z = (int)a.by_ny.div((unsigned)row), y = row - z * a.ny;
+        double fl;
+        dL += f2d(adj_seed_node<P, FLOW>(a, x, y, z, gs, hp, lam, fl));
+        J += fl;
+    }
     const double wL = warp_sum(dL);
     if ((block_thread() & 31) == 0) Lpart[warp_slot()] = wL;
-    const double sJ = block_sum(fl);
+    const double sJ = block_sum(J);
     if (block_thread() == 0) Jpart[block_linear()] = sJ;
 }
 
@@ -2301,7 +2438,13 @@ struct Impl {
     template <int LAYOUT, bool FLOW>
     static void macro_k(const Args& a, const void* f, const void* g, const double* hp,
                         const MacroOut& o, cudaStream_t s) {
-        k_macro<P, LAYOUT, FLOW><<<RED_BLOCKS, RED_THREADS, 0, s>>>(a, (const T*)f, (const TGp*)g, hp, o);
+        // the sums fill RED_BLOCKS partial rows; fields take no more blocks than they have work for
+        const long long need = ((long long)a.N + RED_THREADS - 1) / RED_THREADS;
+        const int blocks = (int)std::min<long long>(need, RED_BLOCKS);
+        if (o.partial)
+            k_macro<P, LAYOUT, FLOW, true><<<RED_BLOCKS, RED_THREADS, 0, s>>>(a, (const T*)f, (const TGp*)g, hp, o);
+        else
+            k_macro<P, LAYOUT, FLOW, false><<<blocks, RED_THREADS, 0, s>>>(a, (const T*)f, (const TGp*)g, hp, o);
     }
     static void macro(const Args& a, Layout lay, const void* f, const void* g, const double* hp,
                       const MacroOut& o, cudaStream_t s) {
@@ -2316,18 +2459,17 @@ struct Impl {
         }
     }
 
+    template <int LAYOUT>
+    static void init_k(const Args& a, const double* Qf, const double* Qg, const double* h0, void* f,
+                       void* g, double* hp, cudaStream_t s) {
+        const auto [grd, blk] = node_grid(a);
+        if (a.flow) k_init<P, LAYOUT, true><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g, hp);
+        else k_init<P, LAYOUT, false><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g, hp);
+    }
     static void init(const Args& a, Layout lay, const double* Qf, const double* Qg,
                      const double* h0, void* f, void* g, double* hp, cudaStream_t s) {
-        const auto [grd, blk] = node_grid(a);
-        if (lay == LAYOUT_PULL) {
-            if (a.flow) k_init<P, LAYOUT_PULL, true><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g);
-            else k_init<P, LAYOUT_PULL, false><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g);
-            k_init_hprime<P, LAYOUT_PULL><<<grd, blk, 0, s>>>(a, Qg, h0, (const TGp*)g, hp);
-        } else {
-            if (a.flow) k_init<P, LAYOUT_AA_NATURAL, true><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g);
-            else k_init<P, LAYOUT_AA_NATURAL, false><<<grd, blk, 0, s>>>(a, Qf, Qg, h0, (T*)f, (TGp*)g);
-            k_init_hprime<P, LAYOUT_AA_NATURAL><<<grd, blk, 0, s>>>(a, Qg, h0, (const TGp*)g, hp);
-        }
+        if (lay == LAYOUT_PULL) init_k<LAYOUT_PULL>(a, Qf, Qg, h0, f, g, hp, s);
+        else init_k<LAYOUT_AA_NATURAL>(a, Qf, Qg, h0, f, g, hp, s);
     }
 
     template <int LAYOUT>
@@ -2353,12 +2495,14 @@ struct Impl {
         else
             step_k<STEP_PULL, 0, true>(a, fs, fd, gs, gd, hp, s, tape_e, tape_m);
     }
-    static void adj_seed(const Args& a, const void* gs, const double* hp, void* lam,
-                         double* Lpart, double* Jpart, cudaStream_t s) {
-        const auto [grd, blk] = node_grid(a);
+    // returns the number of J partials; Lpart (one slot per warp of the node grid) is zero
+    static int adj_seed(const Args& a, const void* gs, const double* hp, void* lam, double* Lpart,
+                        double* Jpart, cudaStream_t s) {
+        const int blocks = std::min(node_grid_blocks(a.nx, a.ny, a.nz), RED_BLOCKS);
         using C = CT<P>;
-        if (a.flow) k_adj_seed<P, true><<<grd, blk, 0, s>>>(a, (const TGp*)gs, hp, (C*)lam, Lpart, Jpart);
-        else k_adj_seed<P, false><<<grd, blk, 0, s>>>(a, (const TGp*)gs, hp, (C*)lam, Lpart, Jpart);
+        if (a.flow) k_adj_seed<P, true><<<blocks, STEP_THREADS, 0, s>>>(a, (const TGp*)gs, hp, (C*)lam, Lpart, Jpart);
+        else k_adj_seed<P, false><<<blocks, STEP_THREADS, 0, s>>>(a, (const TGp*)gs, hp, (C*)lam, Lpart, Jpart);
+        return blocks;
     }
     static void adj_reverse(const Args& a, const void* lin, void* lout, const void* tape_e,
                             const void* tape_m, int wface, double* gtw, double* Lpart,
@@ -2380,7 +2524,8 @@ struct Impl {
 
     static void check(const Args& a, const void* g, const double* hp, int* flag,
                       cudaStream_t s) {
-        k_check<P><<<RED_BLOCKS, 256, 0, s>>>(a, (const TGp*)g, hp, flag);
+        const long long need = ((long long)a.N + 255) / 256;
+        k_check<P><<<(int)std::min<long long>(need, RED_BLOCKS), 256, 0, s>>>(a, (const TGp*)g, hp, flag);
     }
 
     static const Launchers& table() {
