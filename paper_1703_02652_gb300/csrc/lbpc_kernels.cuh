@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "lbpc_internal.h"
 
@@ -242,9 +243,9 @@ template <> LBPC_HD const Coef<double>& coef<double>(const Args& a) { return a.c
     X(5, 0, 0, 1, 6) X(6, 0, 0, -1, 5)
 
 // Neighbour access policies.  Nb: offsets (in nodes) to the neighbours at x-1 / x+1
-// etc. with periodic wrap, and whether that neighbour lies behind a wall.  NbInterior:
-// a node at least one cell away from every face, where every neighbour is a plain
-// constant offset and no wall rule applies.
+// etc. with periodic wrap, and whether that neighbour lies behind a wall.  NbRow: a node of a
+// row away from every y and z face, where only the x rules remain.  NbInterior: the same for
+// a pair kernel's y and z neighbours, which has no rule at all.
 struct Nb {
     int oxm, oxp, oym, oyp, ozm, ozp;
     bool wxm, wxp, wym, wyp, wzm, wzp;
@@ -259,6 +260,17 @@ struct Nb {
         return (EX == 1 && wxm) || (EX == -1 && wxp) || (EY == 1 && wym) || (EY == -1 && wyp) ||
                (EZ == 1 && wzm) || (EZ == -1 && wzp);
     }
+};
+
+struct NbRow {
+    int oxm, oxp, sy, sz;  // x neighbours (with wrap), node strides of y and z
+    bool wxm, wxp;
+    template <int EX, int EY, int EZ>
+    LBPC_HD int off() const {
+        return (EX == 1 ? oxm : EX == -1 ? oxp : 0) - EY * sy - EZ * sz;
+    }
+    template <int EX, int EY, int EZ>
+    LBPC_HD bool wall() const { return (EX == 1 && wxm) || (EX == -1 && wxp); }
 };
 
 struct NbInterior {
@@ -287,8 +299,25 @@ LBPC_HD Nb make_nb(const Args& a, int x, int y, int z) {
     return b;
 }
 
+LBPC_HD NbRow make_nb_row(const Args& a, int x) {
+    return NbRow{x == 0 ? a.nx - 1 : -1, x == a.nx - 1 ? -(a.nx - 1) : 1, a.nx, a.nx * a.ny,
+                 x == 0 && a.wall[0], x == a.nx - 1 && a.wall[1]};
+}
+
+// Row (y, z) away from every y and z face.  The per-node kernels branch on this, which all
+// lanes of most warps agree on; the x rules are selects on two lanes of a row (as a branch they
+// cost the two warps at the ends of every row their gather and scatter twice).
+LBPC_HD bool inner_row(const Args& a, int y, int z) {
+    return y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1;
+}
+
+template <bool FACE>
+LBPC_HD auto inner_nb(const Args& a, int x) {
+    if constexpr (FACE) return NbInterior{a.nx, a.nx * a.ny};
+    else return make_nb_row(a, x);
+}
 LBPC_HD bool is_interior(const Args& a, int x, int y, int z) {
-    return x > 0 && x < a.nx - 1 && y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1;
+    return x > 0 && x < a.nx - 1 && inner_row(a, y, z);
 }
 
 // Index of a node inside the temperature field of face `face`.
@@ -363,27 +392,38 @@ LBPC_HD X ld_any(const X* p) {
     return *p;
 }
 
+// Where a population lies: plane `near` at node m, or behind a wall plane `back` at node n.
+// One offset from the near plane for the rows away from the y and z faces (most of their
+// accesses know at compile time that there is no wall); a plane select on the face rows.
+template <class NB, class X>
+LBPC_HD X* slot_at(X* base, size_t N, int near, int back, bool wall, int n, int m) {
+    if constexpr (!std::is_same_v<NB, NbRow>) {
+        const int idx = wall ? n : m, slot = wall ? back : near;
+        return base + (size_t)slot * N + idx;
+    } else {
+        const ptrdiff_t o = wall ? n + (ptrdiff_t)(back - near) * (ptrdiff_t)N : (ptrdiff_t)m;
+        return base + (size_t)near * N + o;
+    }
+}
+
 template <int P, int LAYOUT, bool HINT, class NB>
 LBPC_HD void gather_f(const Args& a, const NB& b, int n,
                                          const typename Store<P>::T* fs,
                                          typename Store<P>::C* f) {
     using S = Store<P>;
+    using TFt = typename S::T;
     using C = typename S::C;
     const Coef<C>& k = coef<C>(a);
     const size_t N = (size_t)a.N;
 #define LBPC_GF(q, ex, ey, ez, op)                                                       \
     {                                                                                   \
-        int idx;                                                                        \
-        int slot;                                                                       \
-        if constexpr (LAYOUT == LAYOUT_AA_NATURAL) {                                    \
-            idx = n; slot = q;                                                          \
-        } else {                                                                        \
-            const bool w = b.template wall<ex, ey, ez>();                                      \
-            idx = w ? n : n + b.template off<ex, ey, ez>();                                    \
-            if constexpr (LAYOUT == LAYOUT_PULL) slot = w ? op : q;                      \
-            else slot = w ? q : op;                                                     \
-        }                                                                               \
-        f[q] = S::dec(ldv<P, LAYOUT, HINT>(fs + (size_t)slot * N + idx), fshift(k, q));    \
+        constexpr int near = LAYOUT == LAYOUT_AA_SWAPPED ? op : q;  /* slot upwind */     \
+        constexpr int back = LAYOUT == LAYOUT_AA_SWAPPED ? q : op;  /* slot behind a wall */ \
+        const TFt* p = fs + (size_t)q * N + n;                                          \
+        if constexpr (LAYOUT != LAYOUT_AA_NATURAL)                                      \
+            p = slot_at<NB>(fs, N, near, back, b.template wall<ex, ey, ez>(), n,        \
+                            n + b.template off<ex, ey, ez>());                          \
+        f[q] = S::dec(ldv<P, LAYOUT, HINT>(p), fshift(k, q));                           \
     }
     LBPC_Q19(LBPC_GF)
 #undef LBPC_GF
@@ -404,12 +444,12 @@ LBPC_HD void gather_g(const Args& a, const NB& b, int n, int x, int y, int z,
         if constexpr (LAYOUT == LAYOUT_AA_NATURAL) {                                    \
             g[q] = S::dec(ldv<P, LAYOUT, HINT>(gs + (size_t)(q - 1) * N + n), k.gshift);         \
         } else {                                                                        \
-            const bool w = b.template wall<ex, ey, ez>();                                      \
-            const int idx = w ? n : n + b.template off<ex, ey, ez>();                          \
-            int slot;                                                                   \
-            if constexpr (LAYOUT == LAYOUT_PULL) slot = w ? op : q;                      \
-            else slot = w ? q : op;                                                     \
-            C v = S::dec(ldv<P, LAYOUT, HINT>(gs + (size_t)(slot - 1) * N + idx), k.gshift);     \
+            constexpr int near = LAYOUT == LAYOUT_AA_SWAPPED ? op : q;                  \
+            constexpr int back = LAYOUT == LAYOUT_AA_SWAPPED ? q : op;                  \
+            const bool w = b.template wall<ex, ey, ez>();                               \
+            const auto* p = slot_at<NB>(gs, N, near - 1, back - 1, w, n,                \
+                                        n + b.template off<ex, ey, ez>());              \
+            C v = S::dec(ldv<P, LAYOUT, HINT>(p), k.gshift);                            \
             if (w && a.wall_iso[q - 1]) v = S::grid(abb_back(a, k, q - 1, x, y, z, v));   \
             g[q] = v;                                                                   \
         }                                                                               \
@@ -438,8 +478,12 @@ LBPC_HD void scatter_f(const Args& a, const NB& b, int n,
             fd[(size_t)op * N + n] = v;                                                 \
         } else { /* downwind neighbour x + e is the upwind neighbour of -e */           \
             const bool w = b.template wall<-(ex), -(ey), -(ez)>();                             \
-            if (w) fd[(size_t)op * N + n] = v;                                          \
-            else fd[(size_t)q * N + n + b.template off<-(ex), -(ey), -(ez)>()] = v;            \
+            if constexpr (!std::is_same_v<NB, NbRow>) {                                 \
+                if (w) fd[(size_t)op * N + n] = v;                                      \
+                else fd[(size_t)q * N + n + b.template off<-(ex), -(ey), -(ez)>()] = v; \
+            } else {                                                                    \
+                *slot_at<NB>(fd, N, q, op, w, n, n + b.template off<-(ex), -(ey), -(ez)>()) = v; \
+            }                                                                           \
         }                                                                               \
     }
     LBPC_Q19(LBPC_SF)
@@ -851,8 +895,10 @@ template <> struct KindLayout<STEP_AA_EVEN> { static constexpr int value = LAYOU
 template <> struct KindLayout<STEP_AA_ODD> { static constexpr int value = LAYOUT_AA_SWAPPED; };
 
 // One time step of node (x, y, z): gather (stream in, with wall rules), Eq. 2 inversion,
-// flow collision, enthalpy collision, scatter, FP64 rest channel update.
-template <int P, int KIND, int FLOW, bool TAPE = false>
+// flow collision, enthalpy collision, scatter, FP64 rest channel update.  FACE: for the rows
+// that the AA pair kernels leave to it, with the branch on the node's own position (the row
+// form there costs the pair path 1-5% in spills).
+template <int P, int KIND, int FLOW, bool TAPE = false, bool FACE = false>
 LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
                        TF<P>* fd, const TG<P>* gs,
                        TG<P>* gd, double* hp, CT<P>* tape_e = nullptr,
@@ -862,12 +908,12 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     const int n = x + a.nx * (y + a.ny * z);
     constexpr int LAYOUT = KindLayout<KIND>::value;
     constexpr bool HINT = KIND == STEP_PULL;
-    const bool interior = is_interior(a, x, y, z);
-    const NbInterior bi{a.nx, a.nx * a.ny};
+    const bool inner = FACE ? is_interior(a, x, y, z) : inner_row(a, y, z);
+    const auto bi = inner_nb<FACE>(a, x);
     const Nb b = make_nb(a, x, y, z);
 
     C f[19], g[7];
-    if (interior) {
+    if (inner) {
         if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, HINT>(a, bi, n, fs, f);
         gather_g<Mode<P>::G, LAYOUT, HINT>(a, bi, n, x, y, z, gs, g);
     } else {
@@ -892,7 +938,7 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
         }
     }
     collide_enth<C, !FLOW>(g, k, T, fl, ux, uy, uz);
-    if (interior) {
+    if (inner) {
         if constexpr (FLOW) scatter_f<Mode<P>::F, KIND>(a, bi, n, fd, f);
         scatter_g<Mode<P>::G, KIND>(a, bi, n, x, y, z, gd, g);
     } else {
@@ -1084,6 +1130,34 @@ LBPC_HD void step_pair_aa(const Args& a, int x0, int y, int z, TF<P>* F, TG<P>* 
     const int up1 = xhi ? n1 - (a.nx - 1) : n1 + 1;    // x-neighbour x1 + 1 (wrapped)
     C f0[19], f1[19], g0[7], g1[7];
     // ---- gather ----
+    // What is loaded first is a measurement (256 x 256 x 128, us a step): FP16 the rest channel
+    // (182, last 185), FP16 f with FP32 g the g populations (200, last 209).
+    constexpr bool HP_FIRST = P == LBPC_FP16S, G_FIRST = P == LBPC_FP16S_G32;
+    double2 ep;
+    if constexpr (HP_FIRST) ep = *reinterpret_cast<const double2*>(hp + n0);
+#define LBPC_AGG(q, ex, ey, ez, op)                                                      \
+    {                                                                                   \
+        if constexpr (!ODD) {                                                           \
+            PRG::dec(*reinterpret_cast<const VG*>(G + (size_t)(q - 1) * N + n0), k.gshift, g0[q], g1[q]); \
+        } else {                                                                        \
+            const int oyz = -(ey) * sy - (ez) * sz;                                     \
+            const TGt* sw = G + (size_t)(op - 1) * N;                                   \
+            if constexpr ((ex) == 0) {                                                  \
+                PRG::dec(*reinterpret_cast<const VG*>(sw + n0 + oyz), k.gshift, g0[q], g1[q]); \
+            } else if constexpr ((ex) == 1) {                                           \
+                C v = SG::dec(sw[wlo ? ((q) - (op)) * N32 + n0 : dn0 + oyz], k.gshift);  \
+                if (wlo && a.wall_iso[0]) v = SG::grid(-v + abb_source(a, k, 0, x0, y, z)); \
+                g0[q] = v;                                                              \
+                g1[q] = SG::dec(sw[n0 + oyz], k.gshift);                                    \
+            } else {                                                                    \
+                g0[q] = SG::dec(sw[n1 + oyz], k.gshift);                                    \
+                C v = SG::dec(sw[whi ? ((q) - (op)) * N32 + n1 : up1 + oyz], k.gshift);  \
+                if (whi && a.wall_iso[1]) v = SG::grid(-v + abb_source(a, k, 1, x0 + 1, y, z)); \
+                g1[q] = v;                                                              \
+            }                                                                           \
+        }                                                                               \
+    }
+    if constexpr (G_FIRST) { LBPC_Q7(LBPC_AGG) }
     if constexpr (FLOW) {
 #define LBPC_AGF(q, ex, ey, ez, op)                                                      \
         {                                                                               \
@@ -1107,31 +1181,9 @@ LBPC_HD void step_pair_aa(const Args& a, int x0, int y, int z, TF<P>* F, TG<P>* 
         LBPC_Q19(LBPC_AGF)
 #undef LBPC_AGF
     }
-#define LBPC_AGG(q, ex, ey, ez, op)                                                      \
-    {                                                                                   \
-        if constexpr (!ODD) {                                                           \
-            PRG::dec(*reinterpret_cast<const VG*>(G + (size_t)(q - 1) * N + n0), k.gshift, g0[q], g1[q]); \
-        } else {                                                                        \
-            const int oyz = -(ey) * sy - (ez) * sz;                                     \
-            const TGt* sw = G + (size_t)(op - 1) * N;                                   \
-            if constexpr ((ex) == 0) {                                                  \
-                PRG::dec(*reinterpret_cast<const VG*>(sw + n0 + oyz), k.gshift, g0[q], g1[q]); \
-            } else if constexpr ((ex) == 1) {                                           \
-                C v = SG::dec(sw[wlo ? ((q) - (op)) * N32 + n0 : dn0 + oyz], k.gshift);  \
-                if (wlo && a.wall_iso[0]) v = SG::grid(-v + abb_source(a, k, 0, x0, y, z)); \
-                g0[q] = v;                                                              \
-                g1[q] = SG::dec(sw[n0 + oyz], k.gshift);                                    \
-            } else {                                                                    \
-                g0[q] = SG::dec(sw[n1 + oyz], k.gshift);                                    \
-                C v = SG::dec(sw[whi ? ((q) - (op)) * N32 + n1 : up1 + oyz], k.gshift);  \
-                if (whi && a.wall_iso[1]) v = SG::grid(-v + abb_source(a, k, 1, x0 + 1, y, z)); \
-                g1[q] = v;                                                              \
-            }                                                                           \
-        }                                                                               \
-    }
-    LBPC_Q7(LBPC_AGG)
+    if constexpr (!G_FIRST) { LBPC_Q7(LBPC_AGG) }
 #undef LBPC_AGG
-    const double2 ep = *reinterpret_cast<const double2*>(hp + n0);
+    if constexpr (!HP_FIRST) ep = *reinterpret_cast<const double2*>(hp + n0);
     const double e0 = excess_plus<Mode<P>::G>(ep.x, g0), e1 = excess_plus<Mode<P>::G>(ep.y, g1);
     pair_collide<P, FLOW>(a, f0, f1, g0, g1, e0, e1);
     // fresh copies of the indices and bases for the scatter (see opaque())
@@ -1223,8 +1275,8 @@ LBPC_HD void macro_node(const Args& a, int x, int y, int z, const TF<P>* fs, con
     const Coef<C>& k = coef<C>(a);
     const int n = x + a.nx * (y + a.ny * z);
     C f[19], g[7];
-    if (is_interior(a, x, y, z)) {
-        const NbInterior b{a.nx, a.nx * a.ny};
+    if (inner_row(a, y, z)) {
+        const NbRow b = make_nb_row(a, x);
         if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
         gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
     } else {
@@ -1382,8 +1434,8 @@ LBPC_HD void dist_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     const Coef<C>& k = coef<C>(a);
     const bool with_f = FLOW && Qf;
     C f[19], g[7];
-    if (is_interior(a, x, y, z)) {
-        const NbInterior b{a.nx, a.nx * a.ny};
+    if (inner_row(a, y, z)) {
+        const NbRow b = make_nb_row(a, x);
         if (with_f) gather_f<Mode<P>::F, LAYOUT, true>(a, b, n, fs, f);
         gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
     } else {
@@ -1629,8 +1681,8 @@ LBPC_HD CT<P> adj_seed_node(const Args& a, int x, int y, int z,
     const Coef<C>& k = coef<C>(a);
     const int n = x + a.nx * (y + a.ny * z);
     C g[7];
-    if (is_interior(a, x, y, z))
-        gather_g<Mode<P>::G, LAYOUT_PULL, true>(a, NbInterior{a.nx, a.nx * a.ny}, n, x, y, z, gs, g);
+    if (inner_row(a, y, z))
+        gather_g<Mode<P>::G, LAYOUT_PULL, true>(a, make_nb_row(a, x), n, x, y, z, gs, g);
     else
         gather_g<Mode<P>::G, LAYOUT_PULL, true>(a, make_nb(a, x, y, z), n, x, y, z, gs, g);
     const double e = excess_plus<Mode<P>::G>(hp[n], g);
@@ -1663,8 +1715,8 @@ LBPC_HD CT<P> adj_reverse_node(const Args& a, const NB& b, int x, int y, int z,
 #define LBPC_AF(q, ex, ey, ez, op)                                                       \
         {                                                                               \
             const bool w = b.template wall<-(ex), -(ey), -(ez)>();                      \
-            lf[q] = w ? lin[(size_t)op * N + n]                                         \
-                      : lin[(size_t)q * N + n + b.template off<-(ex), -(ey), -(ez)>()];  \
+            lf[q] = lin[(ptrdiff_t)q * a.N + (w ? n + (ptrdiff_t)((op) - (q)) * a.N :    \
+                    (ptrdiff_t)(n + b.template off<-(ex), -(ey), -(ez)>()))];           \
         }
         LBPC_Q19(LBPC_AF)
 #undef LBPC_AF
@@ -1849,8 +1901,12 @@ __device__ __forceinline__ void after_previous_grid(Ptr&... p) {
     if (!item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z)) return;
 
 // One node per thread; with TAPE (pull) also the adjoint tape.
+// Blocks per SM: eight with 32- or 16-bit storage and flow (64 registers): 161 x 161 x 81 FP32
+// 83 us a step, 87 at seven, 92 at nine.
+template <int P, int FLOW>
+constexpr int kNodeBlocks = P == LBPC_FP64 || !FLOW ? 1 : 8;
 template <int P, int KIND, int FLOW, bool TAPE>
-__global__ void __launch_bounds__(STEP_THREADS)
+__global__ void __launch_bounds__(STEP_THREADS, kNodeBlocks<P, FLOW>)
 k_step(const __grid_constant__ Args a, const TF<P>* fs, TF<P>* fd,
        const TG<P>* gs, TG<P>* gd, double* __restrict__ hp, CT<P>* __restrict__ tape_e,
        CT<P>* __restrict__ tape_m) {
@@ -1897,8 +1953,8 @@ k_step_pull_x2(const __grid_constant__ Args a, const TF<P>* fs,
 // the interior path 4% (its registers).
 template <int P, int KIND, int FLOW>
 LBPC_HD void aa_face_pair(const Args& a, int x0, int y, int z, TF<P>* F, TG<P>* G, double* hp) {
-    step_node<P, KIND, FLOW>(a, x0, y, z, F, F, G, G, hp);
-    step_node<P, KIND, FLOW>(a, x0 + 1, y, z, F, F, G, G, hp);
+    step_node<P, KIND, FLOW, false, true>(a, x0, y, z, F, F, G, G, hp);
+    step_node<P, KIND, FLOW, false, true>(a, x0 + 1, y, z, F, F, G, G, hp);
 }
 template <int P, int KIND, int FLOW>
 __device__ __noinline__ void aa_face_pair_call(const Args& a, int x0, int y, int z, TF<P>* F,
@@ -1908,16 +1964,17 @@ __device__ __noinline__ void aa_face_pair_call(const Args& a, int x0, int y, int
 
 // AA step, two nodes per thread along x (even nx); same vote as the pull pair kernel.
 // Five blocks per SM (96 registers; a few bytes of spills in some variants); the even step
-// with 16-bit f six (80 registers; the odd step spills at six).
+// with 16-bit f and g six (80 registers; the odd step spills at six).
 template <int P, int FLOW, bool ODD>
-__global__ void __launch_bounds__(STEP_THREADS, kRebuild<P> && !ODD ? 6 : 5)
+__global__ void __launch_bounds__(STEP_THREADS, sizeof(TG<P>) == 2 && !ODD ? 6 : 5)
 k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* __restrict__ hp) {
+    constexpr bool MIXED = kRebuild<P> && sizeof(TG<P>) == 4;
     int x0, y, z;
     const bool valid = item_cyz(a, a.nx / 2, a.by_hx, a.fill_hx, x0, y, z);
     x0 *= 2;
     const bool inner = !valid || (y > 0 && y < a.ny - 1 && z > 0 && z < a.nz - 1);
-    const bool paired = __all_sync(0xffffffffu, inner);
-    constexpr bool MIXED = kRebuild<P> && sizeof(TG<P>) == 4;
+    // (an even step has no y and z rule; the other modes measured faster with the vote)
+    const bool paired = (MIXED && !ODD) || __all_sync(0xffffffffu, inner);
     if constexpr (MIXED) after_previous_grid(hp);
     else after_previous_grid(F, G);
     if (!valid) return;
@@ -2261,8 +2318,8 @@ k_adj_reverse(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
     const bool valid = item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z);
     after_previous_grid(lin, tape_e, tape_m);
     if (valid) {
-        if (is_interior(a, x, y, z))
-            dL = adj_reverse_node<P, FLOW>(a, NbInterior{a.nx, a.nx * a.ny}, x, y, z, lin, lout,
+        if (inner_row(a, y, z))
+            dL = adj_reverse_node<P, FLOW>(a, make_nb_row(a, x), x, y, z, lin, lout,
                                            tape_e, tape_m, wface, gtw);
         else
             dL = adj_reverse_node<P, FLOW>(a, make_nb(a, x, y, z), x, y, z, lin, lout, tape_e,
@@ -2321,12 +2378,16 @@ inline void launch_after(void (*kern)(K...), const ItemGrid& g, bool early, cuda
     c.numAttrs = early ? 1 : 0;
     cudaLaunchKernelEx(&c, kern, K(args)...);
 }
-// FP64 grids between one warp and six blocks per SM start after the one before instead: early
-// blocks go where that one left room, two to an SM beside idle ones, and share its FP64 pipe
-// (24^3 flow: 35 us a step early, 14.5 after; 8 x 8 x 64: 11.4 and 12.5; 64^3: 153 and 156).
+// FP64 grids of a few blocks per SM start after the one before instead: early blocks go where
+// that one left room, two to an SM beside idle ones, and share its FP64 pipe.  us a step early
+// and after, by blocks of 128 nodes (152 SMs): flow 64 blocks 12.7 / 14.5, 128: 39.8 / 14.5,
+// 384: 43 / 35, 512: 43 / 45, 1024: 73 / 76; conduction 128: 4.9 / 6.2, 192: 9.8 / 7.9, 1036:
+// 18.8 / 17.5, 2048: 25.4 / 26.9.
 template <int P>
 inline bool start_early(const Args& a) {
-    return P != LBPC_FP64 || a.N <= SM_COUNT * 32 || a.N >= 6 * SM_COUNT * STEP_THREADS;
+    const long long blocks = ((long long)a.N + STEP_THREADS - 1) / STEP_THREADS;
+    return P != LBPC_FP64 || blocks <= (a.flow ? SM_COUNT / 2 : SM_COUNT - SM_COUNT / 8) ||
+           blocks >= (a.flow ? 4 : 12) * SM_COUNT;
 }
 inline ItemGrid node_grid(const Args& a) { return item_grid(a.nx, a.ny, a.nz); }
 inline ItemGrid pair_grid(const Args& a) { return item_grid(a.nx / 2, a.ny, a.nz); }
