@@ -15,6 +15,7 @@
 #include "lbpc.h"
 #include "lbpc_host.h"
 #include "lbpc_internal.h"
+#include "lbpc_launch.cuh"
 
 using namespace lbpc;
 
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(256)
 k_finalize(const double* __restrict__ partial, const double* __restrict__ lines, int nx,
            double area, double nu_scale, double fd_scale, double step, int flow, int iso0,
            double* __restrict__ result, double* __restrict__ hist_row) {
+    after_previous_grid(partial, lines);
     __shared__ double sh[256][NRED];
     double acc[NRED] = {0, 0, 0, 0, 0, 0};
     for (int b = threadIdx.x; b < RED_BLOCKS; b += blockDim.x)
@@ -161,8 +163,8 @@ cudaError_t lbpc::finalize_reduction(const double* partial, const double* lines,
                                      double area, double nu_scale, double fd_scale, double step,
                                      int flow, int iso0, double* result, double* hist_row,
                                      cudaStream_t s) {
-    k_finalize<<<1, 256, 0, s>>>(partial, lines, nx, area, nu_scale, fd_scale, step, flow, iso0,
-                                 result, hist_row);
+    launch_after(k_finalize, {dim3(1), dim3(256)}, true, s, partial, lines, nx, area, nu_scale,
+                 fd_scale, step, flow, iso0, result, hist_row);
     return cudaGetLastError();
 }
 
@@ -279,7 +281,9 @@ lbpc_status reset_from_h(lbpc_handle* h, const double* h_host) {
     h->step = 0;
     h->hist_count = 0;
     h->diverged = false;
-    // no diagnostics recorded yet (the workspace comes uninitialised from the caller)
+    // no diagnostics recorded yet, nothing found (the workspace comes uninitialised from the
+    // caller); the flag stays zero until a check sets it, which ends the stepping
+    LBPC_CK(h, cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream));
     LBPC_CK(h, cudaMemsetAsync(h->result, 0, sizeof(double) * LBPC_S_COUNT, h->stream));
     lbpc_status s = init_state(h, nullptr, nullptr, h->stage);
     if (s != LBPC_OK) return s;
@@ -442,7 +446,6 @@ lbpc_status lbpc_step(lbpc_handle* h, int n) {
         // no diagnostics in this mode: check the stored g populations and the FP64 rest
         // channel after the call's last step (a non-finite f reaches g within one step)
         int bad = 0;
-        LBPC_CK(h, cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream));
         h->L->check(h->args, cur_g(h), h->hp, h->flag, h->stream);
         h->launches++;
         LBPC_CK(h, cudaGetLastError());
@@ -546,6 +549,7 @@ lbpc_status lbpc_set_distributions_dev(lbpc_handle* h, const double* f, const do
         return fail(h, LBPC_ERR_STATE, "AA streaming: load a state only after an even step count");
     s = init_state(h, h->p.flow_model != LBPC_FLOW_NONE ? f : nullptr, g, nullptr);
     if (s != LBPC_OK) return s;
+    if (h->diverged) LBPC_CK(h, cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream));
     h->diverged = false;
     return LBPC_OK;
 }
@@ -655,6 +659,7 @@ lbpc_status lbpc_load(lbpc_handle* h, const void* host_buf, size_t bytes) {
         LBPC_CK(h, cudaMemcpy(h->tw[f], o, b, cudaMemcpyHostToDevice));
         o += b;
     }
+    LBPC_CK(h, cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream));
     h->step = hd.step;
     h->hist_count = 0;
     h->diverged = false;

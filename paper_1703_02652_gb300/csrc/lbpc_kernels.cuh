@@ -18,8 +18,7 @@
 #include <type_traits>
 
 #include "lbpc_internal.h"
-
-#define LBPC_HD __host__ __device__ __forceinline__
+#include "lbpc_launch.cuh"
 
 namespace lbpc {
 
@@ -1090,19 +1089,6 @@ LBPC_HD void step_pair_pull(const Args& a, const NB& nb, int x0, int y, int z, c
 }
 
 
-// Hides v's value from the compiler: the scatter addresses of an AA step are gather
-// addresses (the same slots, in place), and without this the compiler keeps them all live
-// across the collision.
-template <class T>
-LBPC_HD void opaque(T& v) {
-#if defined(__CUDA_ARCH__)
-    if constexpr (sizeof(T) == 8) asm volatile("" : "+l"(v));
-    else asm volatile("" : "+r"(v));
-#else
-    (void)v;
-#endif
-}
-
 // AA in-place streaming, two nodes (x0, x0 + 1) per thread, row away from the y/z faces.
 // Even step (natural layout): every access is a local aligned pair; f*_q goes to slot qbar.
 // Odd step (swapped layout): f_q(x) is slot qbar at x - e_q (slot q at x behind a wall) and
@@ -1880,22 +1866,6 @@ __device__ __forceinline__ bool item_cyz(const Args& a, int cols, const FastDiv&
     return y < a.ny;
 }
 
-// In the kernels that follow one another step by step, before any access to their data: lets
-// the next grid of the stream become resident while this one drains, then waits until the
-// previous grid has completed and its stores are visible.  The pointers given go through the
-// barrier: for data that the kernel only reads (const __restrict__) so that no load of it,
-// which the compiler may take for a constant, is moved above; in the pair kernels because the
-// compiler then forms addresses from them after it (which ones is a measurement: up to 8% of a
-// 16-bit step either way).
-// Why: between two dependent launches the GPU waits in steps of about 2 us; 64^3 FP32 took
-// 10.3 us a step without the overlap and 8.0 us with it (6.2 -> 3.1 us at 64 x 1 x 64).
-template <class... Ptr>
-__device__ __forceinline__ void after_previous_grid(Ptr&... p) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    (opaque(p), ...);
-}
-
 #define LBPC_NODE_XYZ                                                                    \
     int x, y, z;                                                                        \
     if (!item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z)) return;
@@ -2171,6 +2141,7 @@ __global__ void __launch_bounds__(RED_THREADS, P == LBPC_FP64 ? 2 : 3)
 k_macro(const __grid_constant__ Args a, const TF<P>* __restrict__ fs,
         const TG<P>* __restrict__ gs, const double* __restrict__ hp,
         const MacroOut out) {
+    after_previous_grid(fs, gs, hp);
     if (SUMS && (long long)blockIdx.x * RED_THREADS >= a.N) {  // no node: a row of zeros
         if (threadIdx.x < NRED) out.partial[blockIdx.x * NRED + threadIdx.x] = 0.0;
         return;
@@ -2248,6 +2219,7 @@ template <int P>
 __global__ void __launch_bounds__(256)
 k_check(const __grid_constant__ Args a, const TG<P>* __restrict__ g,
         const double* __restrict__ hp, int* flag) {
+    after_previous_grid(g, hp);
     int bad = 0;
     const size_t N = (size_t)a.N;
     for (long long n = blockIdx.x * blockDim.x + threadIdx.x; n < a.N;
@@ -2362,22 +2334,6 @@ k_adj_reverse_x2(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
 // ---------------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------------
-// Launch of a kernel that begins with after_previous_grid(): with `early` its blocks may
-// become resident before the stream's previous kernel has completed.
-template <class... K, class... A>
-inline void launch_after(void (*kern)(K...), const ItemGrid& g, bool early, cudaStream_t s,
-                         A... args) {
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c{};
-    c.gridDim = g.grid;
-    c.blockDim = g.block;
-    c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = early ? 1 : 0;
-    cudaLaunchKernelEx(&c, kern, K(args)...);
-}
 // FP64 grids of a few blocks per SM start after the one before instead: early blocks go where
 // that one left room, two to an SM beside idle ones, and share its FP64 pipe.  us a step early
 // and after, by blocks of 128 nodes (152 SMs): flow 64 blocks 12.7 / 14.5, 128: 39.8 / 14.5,
@@ -2503,9 +2459,11 @@ struct Impl {
         const long long need = ((long long)a.N + RED_THREADS - 1) / RED_THREADS;
         const int blocks = (int)std::min<long long>(need, RED_BLOCKS);
         if (o.partial)
-            k_macro<P, LAYOUT, FLOW, true><<<RED_BLOCKS, RED_THREADS, 0, s>>>(a, (const T*)f, (const TGp*)g, hp, o);
+            launch_after(k_macro<P, LAYOUT, FLOW, true>, {dim3(RED_BLOCKS), dim3(RED_THREADS)}, true,
+                         s, a, (const T*)f, (const TGp*)g, hp, o);
         else
-            k_macro<P, LAYOUT, FLOW, false><<<blocks, RED_THREADS, 0, s>>>(a, (const T*)f, (const TGp*)g, hp, o);
+            launch_after(k_macro<P, LAYOUT, FLOW, false>, {dim3(blocks), dim3(RED_THREADS)}, true, s,
+                         a, (const T*)f, (const TGp*)g, hp, o);
     }
     static void macro(const Args& a, Layout lay, const void* f, const void* g, const double* hp,
                       const MacroOut& o, cudaStream_t s) {
@@ -2586,7 +2544,8 @@ struct Impl {
     static void check(const Args& a, const void* g, const double* hp, int* flag,
                       cudaStream_t s) {
         const long long need = ((long long)a.N + 255) / 256;
-        k_check<P><<<(int)std::min<long long>(need, RED_BLOCKS), 256, 0, s>>>(a, (const TGp*)g, hp, flag);
+        launch_after(k_check<P>, {dim3((unsigned)std::min<long long>(need, RED_BLOCKS)), dim3(256)},
+                     true, s, a, (const TGp*)g, hp, flag);
     }
 
     static const Launchers& table() {
