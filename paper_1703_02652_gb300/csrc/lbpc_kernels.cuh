@@ -790,6 +790,177 @@ LBPC_HD void collide_flow(C* f, const Coef<C>& k, C T, C fl, C& ux, C& uy, C& uz
     }
 }
 
+#if defined(__CUDA_ARCH__)
+// ---------------------------------------------------------------------------------
+// FP64 flow collision with its sums in 64-bit integers.
+//
+// GB300 issues one FP64 warp instruction per 16 cycles and SM, whatever it is; of the 300 of a
+// step 230 were additions of the moment transforms.  Populations between 2^-6 and 2^-1 (every
+// state near the rest weights 1/3, 1/18, 1/36) are multiples of 2^-58, so their sums are exact
+// in integers of that unit, two instructions on the integer pipes each; so are the sums of the
+// back-transform in units of 2^-64, to which the corrections d_k are rounded.  What is left to
+// the FP64 pipe are the products.  The error is no larger than of FP64 sums: the moments are
+// exact instead of rounded at each addition, a correction is off by 2^-65 and enters times 30
+// at most (2^-60, against half an ulp of f, 2^-59 to 2^-55), and f* is rounded once.
+// Against quadruple precision, one step from half-melted states: 0.24 ulp rms and 0.6 at most,
+// where FP64 sums gave 0.65 to 0.93 and 4.3.
+// 128^3: 305 FP64 instructions per node and 1110 us a step before, 161 and 537 us now.
+// ---------------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long mantissa_of(unsigned hi, unsigned lo) {
+    return (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
+}
+// f in units of 2^-58; ok: 2^-6 <= f < 2^-1
+__device__ __forceinline__ long long fx_load(double f, bool& ok) {
+    const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
+    ok &= hi - (1017u << 20) < (5u << 20);
+    return (long long)(mantissa_of(hi, lo) << (((hi >> 20) - 1017u) & 7u));
+}
+// the double nearest to m 2^-unit (bits 10 and below of a 64-bit mantissa rounded half up)
+template <int UNIT>
+__device__ __forceinline__ unsigned long long fx_bits(unsigned long long a) {
+    const int n = __clzll((long long)a) & 63;
+    const unsigned long long m = a << n;
+    const unsigned long long b =
+        ((unsigned long long)(1085 - UNIT - n) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+    return a ? b : 0ull;
+}
+__device__ __forceinline__ double fx_double(long long x) {  // units of 2^-58
+    const long long s = x >> 63;
+    const unsigned long long b = fx_bits<58>((unsigned long long)((x ^ s) - s));
+    return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
+}
+// d in units of 2^-64, rounded half up; ok: |d| < 2^-7
+__device__ __forceinline__ long long fx_corr(double d, bool& ok) {
+    const int hi = __double2hiint(d), ex = hi >> 20 & 0x7ff;
+    ok &= ex <= 1015;
+    const unsigned long long m = mantissa_of((unsigned)hi, (unsigned)__double2loint(d)) << 8;
+    const int sh = 1018 - ex;
+    const long long r = (long long)(((m >> (sh < 63 ? sh : 63)) + 1ull) >> 1), s = hi >> 31;
+    return (r ^ s) - s;
+}
+// f* = f + correction, units of 2^-64; ok: 0 < f* < 2^-1
+__device__ __forceinline__ double fx_store(long long f58, long long c64, bool& ok) {
+    const long long v = (f58 << 6) + c64;
+    ok &= v > 0;
+    return __longlong_as_double((long long)fx_bits<64>((unsigned long long)v));
+}
+
+// As collide_flow<false>; false (f is then not to be used) where a value lies outside the
+// ranges above.  No sum overflows within them: the moments stay below 9 x 2^58, the corrections'
+// sums below 42 x 2^57.
+__device__ __forceinline__ bool collide_flow_fx(double* f, const Coef<double>& k, double T,
+                                                double fl, double& ux, double& uy, double& uz,
+                                                double& rho_o, double& jx_o, double& jy_o,
+                                                double& jz_o) {
+    using C = double;
+    using I = long long;
+    bool ok = true;
+    I F[19];
+#pragma unroll
+    for (int q = 0; q < 19; q++) F[q] = fx_load(f[q], ok);
+    const I a1 = F[1] + F[2], b1 = F[1] - F[2];
+    const I a3 = F[3] + F[4], b3 = F[3] - F[4];
+    const I a5 = F[5] + F[6], b5 = F[5] - F[6];
+    const I sxy = (F[7] + F[8]) + (F[9] + F[10]);
+    const I xy_x = (F[7] - F[8]) + (F[9] - F[10]);
+    const I xy_y = (F[7] + F[8]) - (F[9] + F[10]);
+    const C xy_p = fx_double((F[7] - F[8]) - (F[9] - F[10]));
+    const I sxz = (F[11] + F[12]) + (F[13] + F[14]);
+    const I xz_x = (F[11] - F[12]) + (F[13] - F[14]);
+    const I xz_z = (F[11] + F[12]) - (F[13] + F[14]);
+    const C xz_p = fx_double((F[11] - F[12]) - (F[13] - F[14]));
+    const I syz = (F[15] + F[16]) + (F[17] + F[18]);
+    const I yz_y = (F[15] - F[16]) + (F[17] - F[18]);
+    const I yz_z = (F[15] + F[16]) - (F[17] + F[18]);
+    const C yz_p = fx_double((F[15] - F[16]) - (F[17] - F[18]));
+    const I sax = a1 + a3 + a5, sdg = sxy + sxz + syz;
+    const I tx = xy_x + xz_x, ty = xy_y + yz_y, tz = xz_z + yz_z;
+    const C rho = fx_double(F[0] + sax + sdg);
+    const C jx = fx_double(b1 + tx), jy = fx_double(b3 + ty), jz = fx_double(b5 + tz);
+    rho_o = rho;
+    jx_o = jx;
+    jy_o = jy;
+    jz_o = jz;
+    const C m1 = fx_double(sdg - F[0]), m2 = fx_double(9 * F[0] - 7 * sax - 2 * sdg);
+    const C m4 = fx_double(tx - 4 * b1), m6 = fx_double(ty - 4 * b3), m8 = fx_double(tz - 4 * b5);
+    const I a35 = a3 + a5, h9 = (sxy + sxz) - 2 * syz, k11 = sxy - sxz, a53 = a5 - a3;
+    const C m9 = fx_double(2 * a1 - a35 + h9), m10 = fx_double(2 * a35 - 4 * a1 + h9);
+    const C m11 = fx_double(k11 - a53), m12 = fx_double(2 * a53 + k11);
+    const C m16 = fx_double(xy_x - xz_x), m17 = fx_double(yz_y - xy_y), m18 = fx_double(xz_z - yz_z);
+
+    // forces, velocity, equilibrium and corrections as in collide_flow
+    const C Fb = k.gbeta * (T - k.Tref);
+    const C usx = jx, usy = jy, usz = jz + C(0.5) * Fb;
+    const C damp = C(-2) * (C(1) - fl);
+    const C Fx = damp * usx, Fy = damp * usy, Fz = Fb + damp * usz;
+    ux = fl * usx;
+    uy = fl * usy;
+    uz = fl * usz;
+    const C uxx = ux * ux, uyy = uy * uy, uzz = uz * uz, u2 = uxx + uyy + uzz;
+    const C Fu = Fx * ux + Fy * uy + Fz * uz;
+    const C ru2 = rho * u2, rux = rho * ux;
+    const C pxx_eq = rho * (C(3) * uxx - u2), pww_eq = rho * (uyy - uzz);
+    const C FFxx = C(6) * Fx * ux - C(2) * Fu, FFww = C(2) * (Fy * uy - Fz * uz);
+    const C r23 = C(2.0 / 3.0) * rho;
+    const I d1 = fx_corr(k.r_e * (m1 - ru2) + k.c_e * Fu, ok);
+    const I d2 = fx_corr(k.r_eps * (m2 + C(5.5) * ru2) + k.c_eps * Fu, ok);
+    const I d3 = fx_corr(Fx * C(0.1), ok), d5 = fx_corr(Fy * C(0.1), ok),
+            d7 = fx_corr(Fz * C(0.1), ok);
+    const I d4 = fx_corr(k.r_q * (m4 + r23 * ux) + k.c_q * Fx, ok);
+    const I d6 = fx_corr(k.r_q * (m6 + r23 * uy) + k.c_q * Fy, ok);
+    const I d8 = fx_corr(k.r_q * (m8 + r23 * uz) + k.c_q * Fz, ok);
+    const I d9 = fx_corr(k.r_nu9 * (m9 - pxx_eq) + k.c_nu9 * FFxx, ok);
+    const I d10 = fx_corr(k.r_pi10 * (m10 + C(0.5) * pxx_eq) + k.c_pi10 * FFxx, ok);
+    const I d11 = fx_corr(k.r_nu11 * (m11 - pww_eq) + k.c_nu11 * FFww, ok);
+    const I d12 = fx_corr(k.r_pi12 * (m12 + C(0.5) * pww_eq) + k.c_pi12 * FFww, ok);
+    const I d13 = fx_corr(k.r_nu13 * (xy_p - rux * uy) + k.c_nu13 * (Fx * uy + Fy * ux), ok);
+    const I d14 = fx_corr(k.r_nu13 * (yz_p - rho * uy * uz) + k.c_nu13 * (Fy * uz + Fz * uy), ok);
+    const I d15 = fx_corr(k.r_nu13 * (xz_p - rux * uz) + k.c_nu13 * (Fx * uz + Fz * ux), ok);
+    const I d16 = fx_corr(k.r_t * m16, ok), d17 = fx_corr(k.r_t * m17, ok),
+            d18 = fx_corr(k.r_t * m18, ok);
+
+    // back-transform (columns of Eq. 51), sums shared as in collide_flow
+    const I eax = -11 * d1 - 4 * d2, edg = 8 * d1 + d2;
+    f[0] = fx_store(F[0], -30 * d1 + 12 * d2, ok);
+    const I ox = d3 - 4 * d4, oy = d5 - 4 * d6, oz = d7 - 4 * d8;
+    const I ex1 = eax + 2 * d9 - 4 * d10;
+    const I cyz = eax - d9 + 2 * d10, w11 = d11 - 2 * d12;
+    const I ey1 = cyz + w11, ez1 = cyz - w11;
+    f[1] = fx_store(F[1], ex1 + ox, ok);
+    f[2] = fx_store(F[2], ex1 - ox, ok);
+    f[3] = fx_store(F[3], ey1 + oy, ok);
+    f[4] = fx_store(F[4], ey1 - oy, ok);
+    f[5] = fx_store(F[5], ez1 + oz, ok);
+    f[6] = fx_store(F[6], ez1 - oz, ok);
+    const I X = d3 + d4, Y = d5 + d6, Z = d7 + d8;
+    const I a910 = edg + d9 + d10, b1112 = d11 + d12;
+    const I exy = a910 + b1112, exz = a910 - b1112;
+    const I eyz = edg - 2 * d9 - 2 * d10;
+    {
+        const I u = X + d16, v = Y - d17, Pp = exy + d13, Qq = exy - d13;
+        f[7] = fx_store(F[7], Pp + (u + v), ok);
+        f[8] = fx_store(F[8], Qq + (v - u), ok);
+        f[9] = fx_store(F[9], Qq - (v - u), ok);
+        f[10] = fx_store(F[10], Pp - (u + v), ok);
+    }
+    {
+        const I u = X - d16, v = Z + d18, Pp = exz + d15, Qq = exz - d15;
+        f[11] = fx_store(F[11], Pp + (u + v), ok);
+        f[12] = fx_store(F[12], Qq + (v - u), ok);
+        f[13] = fx_store(F[13], Qq - (v - u), ok);
+        f[14] = fx_store(F[14], Pp - (u + v), ok);
+    }
+    {
+        const I u = Y + d17, v = Z - d18, Pp = eyz + d14, Qq = eyz - d14;
+        f[15] = fx_store(F[15], Pp + (u + v), ok);
+        f[16] = fx_store(F[16], Qq + (v - u), ok);
+        f[17] = fx_store(F[17], Qq - (v - u), ok);
+        f[18] = fx_store(F[18], Pp - (u + v), ok);
+    }
+    return ok;
+}
+#endif
+
 // D3Q7 enthalpy collision on the six moving populations (Eq. 21-25; SRT when every
 // rate equals 1/tau_g).  With d_a = g_a - g_a^eq, d_0 = -sum d_a (h is conserved), the
 // moments of d are m1..m3 (odd pairs), m4 = -7 S, m5, m6; g* = g^eq + d - N^-1 R N d.
@@ -897,7 +1068,15 @@ template <> struct KindLayout<STEP_AA_ODD> { static constexpr int value = LAYOUT
 // flow collision, enthalpy collision, scatter, FP64 rest channel update.  FACE: for the rows
 // that the AA pair kernels leave to it, with the branch on the node's own position (the row
 // form there costs the pair path 1-5% in spills).
-template <int P, int KIND, int FLOW, bool TAPE = false, bool FACE = false>
+// FX: FP64 flow collides with integer sums; a node outside their ranges (found before anything
+// is stored) is done again with FP64 sums.
+#if defined(__CUDACC__)
+template <int P, int KIND, int FLOW, bool TAPE>
+__device__ __noinline__ void step_node_fp64(const Args& a, int x, int y, int z, const TF<P>* fs,
+                                            TF<P>* fd, const TG<P>* gs, TG<P>* gd, double* hp,
+                                            CT<P>* tape_e, CT<P>* tape_m);
+#endif
+template <int P, int KIND, int FLOW, bool TAPE = false, bool FACE = false, bool FX = P == LBPC_FP64>
 LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
                        TF<P>* fd, const TG<P>* gs,
                        TG<P>* gd, double* hp, CT<P>* tape_e = nullptr,
@@ -924,9 +1103,18 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     C T, fl;
     invert_excess(a, e, T, fl);
     C ux = C(0), uy = C(0), uz = C(0), rho = C(0), jx = C(0), jy = C(0), jz = C(0);
-    if constexpr (FLOW)  // FLOW 2: the drag closure, phi(f_l) in place of f_l
-        collide_flow<kRebuild<P>>(f, k, T, FLOW == 2 ? darcy_phi(k, fl) : fl, ux, uy, uz, rho, jx,
-                                  jy, jz);
+    if constexpr (FLOW) {  // FLOW 2: the drag closure, phi(f_l) in place of f_l
+        const C phi = FLOW == 2 ? darcy_phi(k, fl) : fl;
+#if defined(__CUDA_ARCH__)
+        if constexpr (FX) {
+            if (!collide_flow_fx(f, k, T, phi, ux, uy, uz, rho, jx, jy, jz)) {
+                step_node_fp64<P, KIND, FLOW, TAPE>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
+                return;
+            }
+        } else
+#endif
+            collide_flow<kRebuild<P>>(f, k, T, phi, ux, uy, uz, rho, jx, jy, jz);
+    }
     if constexpr (TAPE) {  // macroscopic tape of the pre-collision state (adjoint)
         tape_e[n] = tape_excess(a, e, C(0));
         if constexpr (FLOW) {
@@ -946,7 +1134,14 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     }
     hp[n] = excess_minus<Mode<P>::G>(e, g);
 }
-
+#if defined(__CUDACC__)
+template <int P, int KIND, int FLOW, bool TAPE>
+__device__ __noinline__ void step_node_fp64(const Args& a, int x, int y, int z, const TF<P>* fs,
+                                            TF<P>* fd, const TG<P>* gs, TG<P>* gd, double* hp,
+                                            CT<P>* tape_e, CT<P>* tape_m) {
+    step_node<P, KIND, FLOW, TAPE, false, false>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
+}
+#endif
 
 // Inversion and both collisions of a node pair (n0, n0 + 1), in registers; with TAPE also
 // the macroscopic tape of the pair's pre-collision state (adjoint).
@@ -1872,9 +2067,9 @@ __device__ __forceinline__ bool item_cyz(const Args& a, int cols, const FastDiv&
 
 // One node per thread; with TAPE (pull) also the adjoint tape.
 // Blocks per SM: eight with 32- or 16-bit storage and flow (64 registers): 161 x 161 x 81 FP32
-// 83 us a step, 87 at seven, 92 at nine.
+// 83 us a step, 87 at seven, 92 at nine; FP64 flow three: 128^3 537 us, 591 at two.
 template <int P, int FLOW>
-constexpr int kNodeBlocks = P == LBPC_FP64 || !FLOW ? 1 : 8;
+constexpr int kNodeBlocks = !FLOW ? 1 : (P == LBPC_FP64 ? 3 : 8);
 template <int P, int KIND, int FLOW, bool TAPE>
 __global__ void __launch_bounds__(STEP_THREADS, kNodeBlocks<P, FLOW>)
 k_step(const __grid_constant__ Args a, const TF<P>* fs, TF<P>* fd,
@@ -1977,7 +2172,7 @@ constexpr int CL_CTAS = 16;      // one GPC; more than 8 needs the non-portable 
 // path (3-4 us a step, spread over all SMs).  FP64 collisions are bound by the FP64 pipe of
 // the 16 SMs.
 template <int P, bool FLOW>
-constexpr int CL_THREADS = P != LBPC_FP64 ? 512 : (FLOW ? 32 : 256);
+constexpr int CL_THREADS = P == LBPC_FP64 && !FLOW ? 256 : 512;
 
 __device__ __forceinline__ unsigned shared_at(const void* p, unsigned cta) {
     unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
@@ -2392,11 +2587,12 @@ struct Impl {
         }
     }
 
-    // Blocks of steps on one cluster.  Not with 16-bit f or the drag closure: a block of steps has to give the bits of the same
+    // Blocks of steps on one cluster.  Not with FP64 flow (16 SMs' FP64 pipes), and not with
+    // 16-bit f or the drag closure: a block of steps has to give the bits of the same
     // steps one by one, and there the compiler fuses some products of the flow collision
     // otherwise in the loop (a last-bit difference in FP32, which 16-bit storage amplifies).
     static constexpr bool cluster_flow(int flow) {
-        return flow == 0 || (flow == 1 && !kRebuild<P>);
+        return flow == 0 || (flow == 1 && P == LBPC_FP32);
     }
     template <bool FLOW, bool AA>
     static cudaError_t cluster_k(const Args& a, const void* fs, void* fd, const void* gs, void* gd,
