@@ -601,18 +601,95 @@ LBPC_HD C solid_phi(const Coef<C>& k, C fl, C* dphi = nullptr) {
     return fl;
 }
 
-// Density, momentum, Boussinesq force (Eq. 55), solid-phase force -2 (1 - phi) u* and the
-// velocity of Eq. 56 (rho_0 = 1): u = phi (j + F_b / 2), phi = solid_phi(f_l).
+#if defined(__CUDA_ARCH__)
+// ---------------------------------------------------------------------------------
+// FP64 flow collision with its sums in 64-bit integers.
+//
+// GB300 issues one FP64 warp instruction per 16 cycles and SM, whatever it is; of the 300 of a
+// step 230 were additions of the moment transforms.  Populations between 2^-6 and 2^-1 (every
+// state near the rest weights 1/3, 1/18, 1/36) are multiples of 2^-58, so their sums are exact
+// in integers of that unit, two instructions on the integer pipes each; so are the sums of the
+// back-transform in units of 2^-64, to which the corrections d_k are rounded.  What is left to
+// the FP64 pipe are the products.  The error is no larger than of FP64 sums: the moments are
+// exact instead of rounded at each addition, a correction is off by 2^-65 and enters times 30
+// at most (2^-60, against half an ulp of f, 2^-59 to 2^-55), and f* is rounded once.
+// Against quadruple precision, one step from half-melted states: 0.24 ulp rms and 0.6 at most,
+// where FP64 sums gave 0.65 to 0.93 and 4.3.
+// 128^3: 305 FP64 instructions per node and 1110 us a step before, 161 and 537 us now.
+// ---------------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long mantissa_of(unsigned hi, unsigned lo) {
+    return (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
+}
+// f in units of 2^-58; ok: 2^-6 <= f < 2^-1
+__device__ __forceinline__ long long fx_load(double f, bool& ok) {
+    const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
+    ok &= hi - (1017u << 20) < (5u << 20);
+    return (long long)(mantissa_of(hi, lo) << (((hi >> 20) - 1017u) & 7u));
+}
+// the double nearest to m 2^-unit (bits 10 and below of a 64-bit mantissa rounded half up)
+template <int UNIT>
+__device__ __forceinline__ unsigned long long fx_bits(unsigned long long a) {
+    const int n = __clzll((long long)a) & 63;
+    const unsigned long long m = a << n;
+    const unsigned long long b =
+        ((unsigned long long)(1085 - UNIT - n) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+    return a ? b : 0ull;
+}
+__device__ __forceinline__ double fx_double(long long x) {  // units of 2^-58
+    const long long s = x >> 63;
+    const unsigned long long b = fx_bits<58>((unsigned long long)((x ^ s) - s));
+    return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
+}
+// d in units of 2^-64, rounded half up; ok: |d| < 2^-7
+__device__ __forceinline__ long long fx_corr(double d, bool& ok) {
+    const int hi = __double2hiint(d), ex = hi >> 20 & 0x7ff;
+    ok &= ex <= 1015;
+    const unsigned long long m = mantissa_of((unsigned)hi, (unsigned)__double2loint(d)) << 8;
+    const int sh = 1018 - ex;
+    const long long r = (long long)(((m >> (sh < 63 ? sh : 63)) + 1ull) >> 1), s = hi >> 31;
+    return (r ^ s) - s;
+}
+// f* = f + correction, units of 2^-64; ok: 0 < f* < 2^-1
+__device__ __forceinline__ double fx_store(long long f58, long long c64, bool& ok) {
+    const long long v = (f58 << 6) + c64;
+    ok &= v > 0;
+    return __longlong_as_double((long long)fx_bits<64>((unsigned long long)v));
+}
+#endif
+
 template <class C>
-LBPC_HD void flow_macro(const C* f, const Coef<C>& k, C T, C fl, C& rho, C& jx,
-                                           C& jy, C& jz, C& ux, C& uy, C& uz, C& Fx, C& Fy,
-                                           C& Fz) {
+LBPC_HD void flow_sums(const C* f, const Coef<C>& k, C& rho, C& jx, C& jy, C& jz) {
     rho = ((f[0] + (f[1] + f[2])) + ((f[3] + f[4]) + (f[5] + f[6]))) +
           (((f[7] + f[8]) + (f[9] + f[10])) + ((f[11] + f[12]) + (f[13] + f[14])) +
            ((f[15] + f[16]) + (f[17] + f[18]))) + k.frho;
     jx = (f[1] - f[2]) + (f[7] - f[8] + f[9] - f[10]) + (f[11] - f[12] + f[13] - f[14]);
     jy = (f[3] - f[4]) + (f[7] + f[8] - f[9] - f[10]) + (f[15] - f[16] + f[17] - f[18]);
     jz = (f[5] - f[6]) + (f[11] + f[12] - f[13] - f[14]) + (f[15] + f[16] - f[17] - f[18]);
+}
+
+// Density, momentum, Boussinesq force (Eq. 55), solid-phase force -2 (1 - phi) u* and the
+// velocity of Eq. 56 (rho_0 = 1): u = phi (j + F_b / 2), phi = solid_phi(f_l).
+template <class C>
+LBPC_HD void flow_macro(const C* f, const Coef<C>& k, C T, C fl, C& rho, C& jx,
+                                           C& jy, C& jz, C& ux, C& uy, C& uz, C& Fx, C& Fy,
+                                           C& Fz) {
+#if defined(__CUDA_ARCH__)
+    if constexpr (sizeof(C) == 8) {  // integer sums (128^3: 283 us for the fields without)
+        bool ok = true;
+        long long F[19];
+#pragma unroll
+        for (int q = 0; q < 19; q++) F[q] = fx_load(f[q], ok);
+        long long r = F[0];
+#pragma unroll
+        for (int q = 1; q < 19; q++) r += F[q];
+        rho = fx_double(r);
+        jx = fx_double((F[1] - F[2]) + (F[7] - F[8] + F[9] - F[10]) + (F[11] - F[12] + F[13] - F[14]));
+        jy = fx_double((F[3] - F[4]) + (F[7] + F[8] - F[9] - F[10]) + (F[15] - F[16] + F[17] - F[18]));
+        jz = fx_double((F[5] - F[6]) + (F[11] + F[12] - F[13] - F[14]) + (F[15] + F[16] - F[17] - F[18]));
+        if (!ok) flow_sums(f, k, rho, jx, jy, jz);
+    } else
+#endif
+        flow_sums(f, k, rho, jx, jy, jz);
     const C Fb = k.gbeta * (T - k.Tref);
     const C usx = jx, usy = jy, usz = jz + C(0.5) * Fb;
     const C phi = solid_phi(k, fl);
@@ -791,60 +868,6 @@ LBPC_HD void collide_flow(C* f, const Coef<C>& k, C T, C fl, C& ux, C& uy, C& uz
 }
 
 #if defined(__CUDA_ARCH__)
-// ---------------------------------------------------------------------------------
-// FP64 flow collision with its sums in 64-bit integers.
-//
-// GB300 issues one FP64 warp instruction per 16 cycles and SM, whatever it is; of the 300 of a
-// step 230 were additions of the moment transforms.  Populations between 2^-6 and 2^-1 (every
-// state near the rest weights 1/3, 1/18, 1/36) are multiples of 2^-58, so their sums are exact
-// in integers of that unit, two instructions on the integer pipes each; so are the sums of the
-// back-transform in units of 2^-64, to which the corrections d_k are rounded.  What is left to
-// the FP64 pipe are the products.  The error is no larger than of FP64 sums: the moments are
-// exact instead of rounded at each addition, a correction is off by 2^-65 and enters times 30
-// at most (2^-60, against half an ulp of f, 2^-59 to 2^-55), and f* is rounded once.
-// Against quadruple precision, one step from half-melted states: 0.24 ulp rms and 0.6 at most,
-// where FP64 sums gave 0.65 to 0.93 and 4.3.
-// 128^3: 305 FP64 instructions per node and 1110 us a step before, 161 and 537 us now.
-// ---------------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long mantissa_of(unsigned hi, unsigned lo) {
-    return (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
-}
-// f in units of 2^-58; ok: 2^-6 <= f < 2^-1
-__device__ __forceinline__ long long fx_load(double f, bool& ok) {
-    const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
-    ok &= hi - (1017u << 20) < (5u << 20);
-    return (long long)(mantissa_of(hi, lo) << (((hi >> 20) - 1017u) & 7u));
-}
-// the double nearest to m 2^-unit (bits 10 and below of a 64-bit mantissa rounded half up)
-template <int UNIT>
-__device__ __forceinline__ unsigned long long fx_bits(unsigned long long a) {
-    const int n = __clzll((long long)a) & 63;
-    const unsigned long long m = a << n;
-    const unsigned long long b =
-        ((unsigned long long)(1085 - UNIT - n) << 52) + (m >> 11) + ((m >> 10) & 1ull);
-    return a ? b : 0ull;
-}
-__device__ __forceinline__ double fx_double(long long x) {  // units of 2^-58
-    const long long s = x >> 63;
-    const unsigned long long b = fx_bits<58>((unsigned long long)((x ^ s) - s));
-    return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
-}
-// d in units of 2^-64, rounded half up; ok: |d| < 2^-7
-__device__ __forceinline__ long long fx_corr(double d, bool& ok) {
-    const int hi = __double2hiint(d), ex = hi >> 20 & 0x7ff;
-    ok &= ex <= 1015;
-    const unsigned long long m = mantissa_of((unsigned)hi, (unsigned)__double2loint(d)) << 8;
-    const int sh = 1018 - ex;
-    const long long r = (long long)(((m >> (sh < 63 ? sh : 63)) + 1ull) >> 1), s = hi >> 31;
-    return (r ^ s) - s;
-}
-// f* = f + correction, units of 2^-64; ok: 0 < f* < 2^-1
-__device__ __forceinline__ double fx_store(long long f58, long long c64, bool& ok) {
-    const long long v = (f58 << 6) + c64;
-    ok &= v > 0;
-    return __longlong_as_double((long long)fx_bits<64>((unsigned long long)v));
-}
-
 // As collide_flow<false>; false (f is then not to be used) where a value lies outside the
 // ranges above.  No sum overflows within them: the moments stay below 9 x 2^58, the corrections'
 // sums below 42 x 2^57.
@@ -1176,12 +1199,89 @@ LBPC_HD void pair_collide(const Args& a, CT<P>* f0, CT<P>* f1, CT<P>* g0, CT<P>*
     collide_enth<C, !FLOW>(g1, k, T1, fl1, ux1, uy1, uz1);
 }
 
-// Two nodes (x0, x0 + 1), x0 even, of one row: populations with e_x = 0 move as aligned
-// pairs; e_x = +-1 ones are two scalar loads, with the x-face rules (periodic wrap; at a
-// wall the reflected population of the node itself) applied by selecting a 32-bit element
-// offset from the population's plane on the lanes at x = 0 / x = nx - 1; every store is a
-// pair.  The y and z rules are the row's: NbInterior has none (a row away from those
-// faces), Nb selects the wrapped or reflected offset per population.  Requires even nx.
+// Gather of two nodes (x0, x0 + 1), x0 even, of one row in the pull layout: populations with
+// e_x = 0 move as aligned pairs; e_x = +-1 ones are two scalar loads, with the x-face rules
+// (periodic wrap; at a wall the reflected population of the node itself) applied by selecting a
+// 32-bit element offset from the population's plane on the lanes at x = 0 / x = nx - 1.  The y
+// and z rules are the row's: NbInterior has none (a row away from those faces), Nb selects
+// the wrapped or reflected offset per population.  Requires even nx.
+// (As macros over the variables of the two functions that use them: as a function of its own the
+// gather cost the BF16 step 2%.)
+#define LBPC_PF(q, ex, ey, ez, op)                                                       \
+        {                                                                               \
+            const int oyz = nb.template off<0, ey, ez>();                               \
+            const bool w = nb.template wall<0, ey, ez>();                               \
+            const int ob = ((op) - (q)) * N32;  /* the reflected population's plane */    \
+            const C sh = fshift(k, q);                                                  \
+            const TFt* pl = fs + (size_t)q * N;                                           \
+            if constexpr ((ex) == 0) {                                                  \
+                PRF::dec(ld_any<true>(reinterpret_cast<const VF*>(pl + n0 + (w ? ob : oyz))),  \
+                        sh, f0[q], f1[q]);                                              \
+            } else if constexpr ((ex) == 1) {                                           \
+                const int i0 = w || wlo ? ob + n0 : up0 + oyz;                          \
+                f0[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + i0), sh);                 \
+                f1[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + (w ? ob + n1 : n0 + oyz)), sh); \
+            } else {                                                                    \
+                const int i1 = w || whi ? ob + n1 : up1 + oyz;                          \
+                f0[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + (w ? ob + n0 : n1 + oyz)), sh); \
+                f1[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + i1), sh);                 \
+            }                                                                           \
+        }
+#define LBPC_PG(q, ex, ey, ez, op)                                                       \
+    {                                                                                   \
+        const int oyz = nb.template off<0, ey, ez>();                                   \
+        const bool w = nb.template wall<0, ey, ez>();                                   \
+        const int ob = ((op) - (q)) * N32;                                              \
+        const TGt* pl = gs + (size_t)(q - 1) * N;                                         \
+        if constexpr ((ex) == 0) {                                                      \
+            PRG::dec(ld_any<true>(reinterpret_cast<const VG*>(pl + n0 + (w ? ob : oyz))),      \
+                    k.gshift, g0[q], g1[q]);                                            \
+            if (w && a.wall_iso[q - 1]) {                                               \
+                g0[q] = SG::grid(-g0[q] + abb_source(a, k, q - 1, x0, y, z));           \
+                g1[q] = SG::grid(-g1[q] + abb_source(a, k, q - 1, x0 + 1, y, z));       \
+            }                                                                           \
+        } else if constexpr ((ex) == 1) {                                               \
+            const int i0 = wlo ? ob + n0 : up0 + oyz;                                   \
+            C v = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + i0), k.gshift);                 \
+            if (wlo && a.wall_iso[0]) v = SG::grid(-v + abb_source(a, k, 0, x0, y, z)); \
+            g0[q] = v;                                                                  \
+            g1[q] = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + n0 + oyz), k.gshift);         \
+        } else {                                                                        \
+            const int i1 = whi ? ob + n1 : up1 + oyz;                                   \
+            C v = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + i1), k.gshift);                 \
+            if (whi && a.wall_iso[1]) v = SG::grid(-v + abb_source(a, k, 1, x0 + 1, y, z)); \
+            g1[q] = v;                                                                  \
+            g0[q] = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + n1 + oyz), k.gshift);         \
+        }                                                                               \
+    }
+template <int P, bool FLOW, class NB>
+LBPC_HD void gather_pair_pull(const Args& a, const NB& nb, int x0, int y, int z, const TF<P>* fs,
+                              const TG<P>* gs, const double* hp, CT<P>* f0, CT<P>* f1, CT<P>* g0,
+                              CT<P>* g1, double2& ep) {
+    using SF = Store<Mode<P>::F>;
+    using SG = Store<Mode<P>::G>;
+    using TFt = typename SF::T;
+    using TGt = typename SG::T;
+    using C = CT<P>;
+    using VF = typename Vec2<TFt>::type;
+    using VG = typename Vec2<TGt>::type;
+    using PRF = Pair<Mode<P>::F>;
+    using PRG = Pair<Mode<P>::G>;
+    const Coef<C>& k = coef<C>(a);
+    const size_t N = (size_t)a.N;
+    const int N32 = a.N;  // 3 N < 2^31 (kPairMaxN)
+    const int n0 = x0 + a.nx * (y + a.ny * z), n1 = n0 + 1;
+    const bool xlo = x0 == 0, xhi = x0 + 1 == a.nx - 1;
+    const bool wlo = xlo && a.wall[0], whi = xhi && a.wall[1];
+    // upwind x-neighbour of node 0 for e_x = +1 and of node 1 for e_x = -1 (with wrap)
+    const int up0 = xlo ? n0 + a.nx - 1 : n0 - 1;
+    const int up1 = xhi ? n1 - (a.nx - 1) : n1 + 1;
+    if constexpr (FLOW) { LBPC_Q19(LBPC_PF) }
+    LBPC_Q7(LBPC_PG)
+    ep = *reinterpret_cast<const double2*>(hp + n0);
+}
+
+// One time step of such a pair; every store is a pair.
 template <int P, int FLOW, bool TAPE, class NB>
 LBPC_HD void step_pair_pull(const Args& a, const NB& nb, int x0, int y, int z, const TF<P>* fs,
                             TF<P>* fd, const TG<P>* gs,
@@ -1210,59 +1310,8 @@ LBPC_HD void step_pair_pull(const Args& a, const NB& nb, int x0, int y, int z, c
     constexpr bool EARLY = Store<Mode<P>::G>::kGrid;
     double2 ep;
     if constexpr (EARLY) ep = *reinterpret_cast<const double2*>(hp + n0);
-    if constexpr (FLOW) {
-#define LBPC_PF(q, ex, ey, ez, op)                                                       \
-        {                                                                               \
-            const int oyz = nb.template off<0, ey, ez>();                               \
-            const bool w = nb.template wall<0, ey, ez>();                               \
-            const int ob = ((op) - (q)) * N32;  /* the reflected population's plane */    \
-            const C sh = fshift(k, q);                                                  \
-            const TFt* pl = fs + (size_t)q * N;                                           \
-            if constexpr ((ex) == 0) {                                                  \
-                PRF::dec(ld_any<true>(reinterpret_cast<const VF*>(pl + n0 + (w ? ob : oyz))),  \
-                        sh, f0[q], f1[q]);                                              \
-            } else if constexpr ((ex) == 1) {                                           \
-                const int i0 = w || wlo ? ob + n0 : up0 + oyz;                          \
-                f0[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + i0), sh);                 \
-                f1[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + (w ? ob + n1 : n0 + oyz)), sh); \
-            } else {                                                                    \
-                const int i1 = w || whi ? ob + n1 : up1 + oyz;                          \
-                f0[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + (w ? ob + n0 : n1 + oyz)), sh); \
-                f1[q] = SF::dec(ldv<Mode<P>::F, LAYOUT_PULL, true>(pl + i1), sh);                 \
-            }                                                                           \
-        }
-        LBPC_Q19(LBPC_PF)
-#undef LBPC_PF
-    }
-#define LBPC_PG(q, ex, ey, ez, op)                                                       \
-    {                                                                                   \
-        const int oyz = nb.template off<0, ey, ez>();                                   \
-        const bool w = nb.template wall<0, ey, ez>();                                   \
-        const int ob = ((op) - (q)) * N32;                                              \
-        const TGt* pl = gs + (size_t)(q - 1) * N;                                         \
-        if constexpr ((ex) == 0) {                                                      \
-            PRG::dec(ld_any<true>(reinterpret_cast<const VG*>(pl + n0 + (w ? ob : oyz))),      \
-                    k.gshift, g0[q], g1[q]);                                            \
-            if (w && a.wall_iso[q - 1]) {                                               \
-                g0[q] = SG::grid(-g0[q] + abb_source(a, k, q - 1, x0, y, z));           \
-                g1[q] = SG::grid(-g1[q] + abb_source(a, k, q - 1, x0 + 1, y, z));       \
-            }                                                                           \
-        } else if constexpr ((ex) == 1) {                                               \
-            const int i0 = wlo ? ob + n0 : up0 + oyz;                                   \
-            C v = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + i0), k.gshift);                 \
-            if (wlo && a.wall_iso[0]) v = SG::grid(-v + abb_source(a, k, 0, x0, y, z)); \
-            g0[q] = v;                                                                  \
-            g1[q] = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + n0 + oyz), k.gshift);         \
-        } else {                                                                        \
-            const int i1 = whi ? ob + n1 : up1 + oyz;                                   \
-            C v = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + i1), k.gshift);                 \
-            if (whi && a.wall_iso[1]) v = SG::grid(-v + abb_source(a, k, 1, x0 + 1, y, z)); \
-            g1[q] = v;                                                                  \
-            g0[q] = SG::dec(ldv<Mode<P>::G, LAYOUT_PULL, true>(pl + n1 + oyz), k.gshift);         \
-        }                                                                               \
-    }
+    if constexpr (FLOW) { LBPC_Q19(LBPC_PF) }
     LBPC_Q7(LBPC_PG)
-#undef LBPC_PG
     if constexpr (!EARLY) ep = *reinterpret_cast<const double2*>(hp + n0);
     const double e0 = excess_plus<Mode<P>::G>(ep.x, g0), e1 = excess_plus<Mode<P>::G>(ep.y, g1);
     pair_collide<P, FLOW, TAPE>(a, f0, f1, g0, g1, e0, e1, n0, tape_e, tape_m);
@@ -1283,6 +1332,9 @@ LBPC_HD void step_pair_pull(const Args& a, const NB& nb, int x0, int y, int z, c
     *reinterpret_cast<double2*>(hp + n0) = make_double2(excess_minus<Mode<P>::G>(e0, g0), excess_minus<Mode<P>::G>(e1, g1));
 }
 
+
+#undef LBPC_PF
+#undef LBPC_PG
 
 // AA in-place streaming, two nodes (x0, x0 + 1) per thread, row away from the y/z faces.
 // Even step (natural layout): every access is a local aligned pair; f*_q goes to slot qbar.
@@ -1447,13 +1499,69 @@ struct MacroSums {
 __device__ __noinline__ inline void add_mushy(double& fl, double e, double L_inv) { fl += e * L_inv; }
 #endif
 
-// Macroscopic state of node (x, y, z): with SUMS its contributions to the diagnostics sums and
-// the front lines, otherwise its fields.
+// Contributions of node (x, y, z), gathered populations f and g and excess e, to the diagnostics
+// sums and the front lines.
+template <int P, bool FLOW>
+LBPC_HD void macro_sums(const Args& a, int x, int y, int z, const CT<P>* f, const CT<P>* g, double e,
+                        const MacroOut& out, MacroSums& acc) {
+    using C = CT<P>;
+    const Coef<C>& k = coef<C>(a);
+    C rho = C(0);
+    if constexpr (FLOW) {
+        C T, fl, jx, jy, jz, ux, uy, uz, Fx, Fy, Fz;  // only rho is used
+        invert_excess(a, e, T, fl);
+        flow_macro(f, k, T, fl, rho, jx, jy, jz, ux, uy, uz, Fx, Fy, Fz);
+    }
+#if defined(__CUDA_ARCH__)
+    const Phase ph = phase_of(e, a.cd.L);
+    if (ph.liquid) acc.liquid++;
+    else if (!ph.solid) add_mushy(acc.fl, e, a.cd.L_inv);
+    acc.nodes++;
+    acc.e += e;
+    if constexpr (FLOW) acc.rho += f2d(rho);
+    if (x == 0 || y == a.ny / 2) {
+        double Td, fld;
+        invert_excess(a, e, Td, fld);
+        if (x == 0) {
+            const double Tw = a.Tw[0][y + a.ny * z];
+            if (a.wall_iso[0])
+                acc.flux += 2.0 * (f2d(g[1]) + f2d(k.gshift)) - f2d(k.wT_cref) * Tw;
+            acc.grad += (Tw - Td) * 2.0;
+        }
+        if (y == a.ny / 2) {
+            if (z == a.nz / 4) out.lines[x] = fld;
+            if (z == a.nz / 2) out.lines[a.nx + x] = fld;
+            if (z == (3 * a.nz) / 4) out.lines[2 * a.nx + x] = fld;
+        }
+    }
+    const C gsum = ((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]);
+    if (not_finite(e) || not_finite(rho) || not_finite(gsum)) acc.bad++;
+#endif
+}
+
+// The fields of a node (T, f_l, h, rho, u) from its gathered populations and excess.
+template <int P, bool FLOW>
+LBPC_HD void macro_fields(const Args& a, const CT<P>* f, double e, double* v) {
+    using C = CT<P>;
+    invert_excess(a, e, v[0], v[1]);  // the FP64 inversion
+    v[2] = a.hs + e;
+    C rho = C(0), ux = C(0), uy = C(0), uz = C(0);
+    if constexpr (FLOW) {  // the velocity as the step computes it
+        C T, fl, jx, jy, jz, Fx, Fy, Fz;
+        invert_excess(a, e, T, fl);
+        flow_macro(f, coef<C>(a), T, fl, rho, jx, jy, jz, ux, uy, uz, Fx, Fy, Fz);
+    }
+    v[3] = f2d(rho);
+    v[4] = f2d(ux);
+    v[5] = f2d(uy);
+    v[6] = f2d(uz);
+}
+
+// Node (x, y, z): with SUMS its contributions to the diagnostics, otherwise its fields.
 template <int P, int LAYOUT, bool FLOW, bool SUMS>
 LBPC_HD void macro_node(const Args& a, int x, int y, int z, const TF<P>* fs, const TG<P>* gs,
                         const double* hp, const MacroOut& out, MacroSums& acc) {
     using C = CT<P>;
-    const Coef<C>& k = coef<C>(a);
     const int n = x + a.nx * (y + a.ny * z);
     C f[19], g[7];
     if (inner_row(a, y, z)) {
@@ -1466,48 +1574,44 @@ LBPC_HD void macro_node(const Args& a, int x, int y, int z, const TF<P>* fs, con
         gather_g<Mode<P>::G, LAYOUT, true>(a, b, n, x, y, z, gs, g);
     }
     const double e = excess_plus<Mode<P>::G>(hp[n], g);
-    C rho = C(0), ux = C(0), uy = C(0), uz = C(0);
-    if constexpr (FLOW) {  // the velocity as the step computes it
-        C T, fl, jx, jy, jz, Fx, Fy, Fz;
-        invert_excess(a, e, T, fl);
-        flow_macro(f, k, T, fl, rho, jx, jy, jz, ux, uy, uz, Fx, Fy, Fz);
-    }
-    if constexpr (!SUMS) {
-        double Td, fld;  // the FP64 inversion
-        invert_excess(a, e, Td, fld);
-        if (out.T) out.T[n] = Td;
-        if (out.fl) out.fl[n] = fld;
-        if (out.h) out.h[n] = a.hs + e;
-        if (out.rho) out.rho[n] = f2d(rho);
-        if (out.ux) out.ux[n] = f2d(ux);
-        if (out.uy) out.uy[n] = f2d(uy);
-        if (out.uz) out.uz[n] = f2d(uz);
+    if constexpr (SUMS) {
+        macro_sums<P, FLOW>(a, x, y, z, f, g, e, out, acc);
     } else {
-#if defined(__CUDACC__)
-        const Phase ph = phase_of(e, a.cd.L);
-        if (ph.liquid) acc.liquid++;
-        else if (!ph.solid) add_mushy(acc.fl, e, a.cd.L_inv);
-        acc.nodes++;
-        acc.e += e;
-        if constexpr (FLOW) acc.rho += f2d(rho);
-        if (x == 0 || y == a.ny / 2) {
-            double Td, fld;
-            invert_excess(a, e, Td, fld);
-            if (x == 0) {
-                const double Tw = a.Tw[0][y + a.ny * z];
-                if (a.wall_iso[0])
-                    acc.flux += 2.0 * (f2d(g[1]) + f2d(k.gshift)) - f2d(k.wT_cref) * Tw;
-                acc.grad += (Tw - Td) * 2.0;
-            }
-            if (y == a.ny / 2) {
-                if (z == a.nz / 4) out.lines[x] = fld;
-                if (z == a.nz / 2) out.lines[a.nx + x] = fld;
-                if (z == (3 * a.nz) / 4) out.lines[2 * a.nx + x] = fld;
-            }
-        }
-        const C gsum = ((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]);
-        if (not_finite(e) || not_finite(rho) || not_finite(gsum)) acc.bad++;
-#endif
+        double v[7];
+        macro_fields<P, FLOW>(a, f, e, v);
+        double* const o[7] = {out.T, out.fl, out.h, out.rho, out.ux, out.uy, out.uz};
+#pragma unroll
+        for (int i = 0; i < 7; i++)
+            if (o[i]) o[i][n] = v[i];
+    }
+}
+
+// The same for a node pair of the pull layout (even nx), fields stored as pairs (16-byte
+// aligned outputs).
+template <int P, bool FLOW, bool SUMS>
+LBPC_HD void macro_pair(const Args& a, int x0, int y, int z, const TF<P>* fs, const TG<P>* gs,
+                        const double* hp, const MacroOut& out, MacroSums& acc) {
+    using C = CT<P>;
+    const int n0 = x0 + a.nx * (y + a.ny * z);
+    C f0[19], f1[19], g0[7], g1[7];
+    double2 ep;
+    if (inner_row(a, y, z))
+        gather_pair_pull<P, FLOW>(a, NbInterior{a.nx, a.nx * a.ny}, x0, y, z, fs, gs, hp, f0, f1, g0,
+                                  g1, ep);
+    else
+        gather_pair_pull<P, FLOW>(a, make_nb(a, x0, y, z), x0, y, z, fs, gs, hp, f0, f1, g0, g1, ep);
+    const double e0 = excess_plus<Mode<P>::G>(ep.x, g0), e1 = excess_plus<Mode<P>::G>(ep.y, g1);
+    if constexpr (SUMS) {
+        macro_sums<P, FLOW>(a, x0, y, z, f0, g0, e0, out, acc);
+        macro_sums<P, FLOW>(a, x0 + 1, y, z, f1, g1, e1, out, acc);
+    } else {
+        double v[7], w[7];
+        macro_fields<P, FLOW>(a, f0, e0, v);
+        macro_fields<P, FLOW>(a, f1, e1, w);
+        double* const o[7] = {out.T, out.fl, out.h, out.rho, out.ux, out.uy, out.uz};
+#pragma unroll
+        for (int i = 0; i < 7; i++)
+            if (o[i]) *reinterpret_cast<double2*>(o[i] + n0) = make_double2(v[i], w[i]);
     }
 }
 
@@ -2330,24 +2434,34 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 // Macroscopic fields of the current state, or (SUMS) FP64 block partial sums for diagnostics:
-// grid-stride over nodes, one partial row per block, summed later in a fixed order.
-template <int P, int LAYOUT, bool FLOW, bool SUMS>
-__global__ void __launch_bounds__(RED_THREADS, P == LBPC_FP64 ? 2 : 3)
+// grid-stride over nodes, or over node pairs (PAIR: pull layout, even nx), one partial row per
+// block, summed later in a fixed order.  Pairs halve the loads of the populations that move
+// with e_x = 0.  us of a read at 256^3, nodes and pairs: fields FP32 578 and 430, FP16 593 and
+// 364, scalars FP32 542 and 375, FP16 597 and 331.
+template <int P, int LAYOUT, bool FLOW, bool SUMS, bool PAIR>
+__global__ void __launch_bounds__(RED_THREADS, P == LBPC_FP64 || PAIR ? 2 : 3)
 k_macro(const __grid_constant__ Args a, const TF<P>* __restrict__ fs,
         const TG<P>* __restrict__ gs, const double* __restrict__ hp,
         const MacroOut out) {
     after_previous_grid(fs, gs, hp);
-    if (SUMS && (long long)blockIdx.x * RED_THREADS >= a.N) {  // no node: a row of zeros
+    const int items = PAIR ? a.N / 2 : a.N;
+    if (SUMS && (long long)blockIdx.x * RED_THREADS >= items) {  // no node: a row of zeros
         if (threadIdx.x < NRED) out.partial[blockIdx.x * NRED + threadIdx.x] = 0.0;
         return;
     }
     MacroSums m{};
     // 64-bit loop index: n + stride may pass 2^31 - 1 near the node limit
-    for (long long n = blockIdx.x * blockDim.x + threadIdx.x; n < a.N;
+    for (long long n = blockIdx.x * blockDim.x + threadIdx.x; n < items;
          n += (long long)gridDim.x * blockDim.x) {
-        const int row = (int)a.by_nx.div((unsigned)n), x = (int)n - row * a.nx;
-        const int z = (int)a.by_ny.div((unsigned)row), y = row - z * a.ny;
-        macro_node<P, LAYOUT, FLOW, SUMS>(a, x, y, z, fs, gs, hp, out, m);
+        if constexpr (PAIR) {
+            const int row = (int)a.by_hx.div((unsigned)n), c = (int)n - row * (a.nx / 2);
+            const int z = (int)a.by_ny.div((unsigned)row), y = row - z * a.ny;
+            macro_pair<P, FLOW, SUMS>(a, 2 * c, y, z, fs, gs, hp, out, m);
+        } else {
+            const int row = (int)a.by_nx.div((unsigned)n), x = (int)n - row * a.nx;
+            const int z = (int)a.by_ny.div((unsigned)row), y = row - z * a.ny;
+            macro_node<P, LAYOUT, FLOW, SUMS>(a, x, y, z, fs, gs, hp, out, m);
+        }
     }
     if constexpr (SUMS) {
         // tree over the block in shared memory: a third of the FP64 operations of warp shuffles
@@ -2648,18 +2762,30 @@ struct Impl {
         return cluster_f(a, aa, fs, fd, gs, gd, hp, n, odd, nullptr, s);
     }
 
+    template <int LAYOUT, bool FLOW, bool SUMS, bool PAIR>
+    static void macro_l(const Args& a, int items, const void* f, const void* g, const double* hp,
+                        const MacroOut& o, cudaStream_t s) {
+        // the sums fill RED_BLOCKS partial rows; fields take no more blocks than they have work for
+        const long long need = ((long long)items + RED_THREADS - 1) / RED_THREADS;
+        const int blocks = SUMS ? RED_BLOCKS : (int)std::min<long long>(need, RED_BLOCKS);
+        launch_after(k_macro<P, LAYOUT, FLOW, SUMS, PAIR>, {dim3(blocks), dim3(RED_THREADS)}, true, s,
+                     a, (const T*)f, (const TGp*)g, hp, o);
+    }
     template <int LAYOUT, bool FLOW>
     static void macro_k(const Args& a, const void* f, const void* g, const double* hp,
                         const MacroOut& o, cudaStream_t s) {
-        // the sums fill RED_BLOCKS partial rows; fields take no more blocks than they have work for
-        const long long need = ((long long)a.N + RED_THREADS - 1) / RED_THREADS;
-        const int blocks = (int)std::min<long long>(need, RED_BLOCKS);
-        if (o.partial)
-            launch_after(k_macro<P, LAYOUT, FLOW, true>, {dim3(RED_BLOCKS), dim3(RED_THREADS)}, true,
-                         s, a, (const T*)f, (const TGp*)g, hp, o);
-        else
-            launch_after(k_macro<P, LAYOUT, FLOW, false>, {dim3(blocks), dim3(RED_THREADS)}, true, s,
-                         a, (const T*)f, (const TGp*)g, hp, o);
+        if constexpr (P != LBPC_FP64 && LAYOUT == LAYOUT_PULL) {
+            bool pairs = a.nx % 2 == 0 && a.N <= kPairMaxN;
+            for (double* v : {o.T, o.fl, o.h, o.rho, o.ux, o.uy, o.uz})
+                pairs = pairs && ((uintptr_t)v & 15) == 0;  // the caller's arrays
+            if (pairs) {
+                if (o.partial) macro_l<LAYOUT, FLOW, true, true>(a, a.N / 2, f, g, hp, o, s);
+                else macro_l<LAYOUT, FLOW, false, true>(a, a.N / 2, f, g, hp, o, s);
+                return;
+            }
+        }
+        if (o.partial) macro_l<LAYOUT, FLOW, true, false>(a, a.N, f, g, hp, o, s);
+        else macro_l<LAYOUT, FLOW, false, false>(a, a.N, f, g, hp, o, s);
     }
     static void macro(const Args& a, Layout lay, const void* f, const void* g, const double* hp,
                       const MacroOut& o, cudaStream_t s) {
