@@ -132,11 +132,10 @@ struct Launchers {
 };
 
 // Launch shape of the kernels that give each node (cols = nx) or node pair (cols = nx / 2)
-// a thread, in blocks of STEP_THREADS: whole rows where they fill blocks, otherwise items
-// counted in memory order (see item_cyz).  With planes of less
-// than eight blocks the count runs through the whole lattice (a second division per thread)
-// instead of starting anew at each z.  (Blocks of 32 or 64 on small lattices measured the
-// same: the step's latency does not depend on them.)
+// a thread, in blocks of t: whole rows where they fill blocks, otherwise items counted in
+// memory order (see item_cyz).  With planes of less than eight blocks the count runs through
+// the whole lattice (a second division per thread) instead of starting anew at each z.
+// (Smaller blocks on small lattices gain nothing but in FP64, see step_grid.)
 constexpr int SM_COUNT = 152;
 // rows_fill: rows of cols items (with ny of them in a plane) fill whole blocks.
 struct ItemGrid { dim3 grid, block; };
@@ -145,11 +144,10 @@ inline bool rows_fill(int cols, int ny) {
     if (cols % STEP_THREADS != 0 && (STEP_THREADS % cols != 0 || cols < 8)) return false;
     return ny % block_rows(cols) == 0 || ny >= 8 * block_rows(cols);
 }
-inline ItemGrid item_grid(int cols, int ny, int nz) {
+inline ItemGrid item_grid(int cols, int ny, int nz, int t = STEP_THREADS) {
     const long long plane = (long long)cols * ny, all = plane * nz;
-    constexpr int t = STEP_THREADS;
     if (rows_fill(cols, ny)) {
-        const int by = block_rows(cols), bx = t / by;
+        const int bx = cols < t ? cols : t, by = t / bx;
         return {dim3(cols / bx, (ny + by - 1) / by, nz), dim3(bx, by)};
     }
     if (plane < 8 * t || nz == 1) return {dim3((unsigned)((all + t - 1) / t)), dim3(t)};

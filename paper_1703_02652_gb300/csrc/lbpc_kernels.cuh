@@ -2155,14 +2155,15 @@ __device__ __forceinline__ bool item_cyz(const Args& a, int cols, const FastDiv&
     const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned row = by_cols.div(p);
     c = (int)(p - row * (unsigned)cols);
+    const bool in = (int)p >= 0;  // (the last block may pass 2^31 - 1, where div ends)
     if (gridDim.y == 1) {
         z = (int)a.by_ny.div(row);
         y = (int)row - z * a.ny;
-        return z < a.nz;
+        return in && z < a.nz;
     }
     z = blockIdx.y;
     y = (int)row;
-    return y < a.ny;
+    return in && y < a.ny;
 }
 
 #define LBPC_NODE_XYZ                                                                    \
@@ -2643,16 +2644,24 @@ k_adj_reverse_x2(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
 // ---------------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------------
-// FP64 grids of a few blocks per SM start after the one before instead: early blocks go where
-// that one left room, two to an SM beside idle ones, and share its FP64 pipe.  us a step early
-// and after, by blocks of 128 nodes (152 SMs): flow 64 blocks 12.7 / 14.5, 128: 39.8 / 14.5,
-// 384: 43 / 35, 512: 43 / 45, 1024: 73 / 76; conduction 128: 4.9 / 6.2, 192: 9.8 / 7.9, 1036:
-// 18.8 / 17.5, 2048: 25.4 / 26.9.
+// FP64 lattices.  Grids of some warps per SM start after the one before instead: early blocks go
+// where that one left room, several to an SM beside idle ones, and share its FP64 pipe.  Blocks
+// of one warp spread best until there are many per SM.  us a step, early / after with 32 threads
+// a block, the better of the two with 128:
+//   flow, nodes       4096: 9.0 / 10.3, 9.3    8192: 13.3 / 10.3, 10.4   24,576: 18.1 / 13.1, 15.9
+//                   49,152: 18.7 / 18.6, 18.7   65,536: 23.8 / 26.7, 24.0  262,144: 74 / 76, 73
+//   conduction       8192: 3.7 / 6.2, 4.1    16,384: 4.6 / 6.2, 5.4    24,576: 11.5 / 6.3, 7.8
+//                   98,735: 15.5 / 14.4, 14.4  262,144: 25.2 / 26.7, 25.4
 template <int P>
 inline bool start_early(const Args& a) {
-    const long long blocks = ((long long)a.N + STEP_THREADS - 1) / STEP_THREADS;
-    return P != LBPC_FP64 || blocks <= (a.flow ? SM_COUNT / 2 : SM_COUNT - SM_COUNT / 8) ||
-           blocks >= (a.flow ? 4 : 12) * SM_COUNT;
+    if (P != LBPC_FP64) return true;
+    return a.flow ? a.N <= 32 * SM_COUNT || a.N >= 3 * STEP_THREADS * SM_COUNT
+                  : a.N <= 112 * SM_COUNT || a.N >= 12 * STEP_THREADS * SM_COUNT;
+}
+template <int P>
+inline ItemGrid step_grid(const Args& a) {
+    const bool one_warp = P == LBPC_FP64 && a.N < 7 * STEP_THREADS * SM_COUNT;
+    return item_grid(a.nx, a.ny, a.nz, one_warp ? 32 : STEP_THREADS);
 }
 inline ItemGrid node_grid(const Args& a) { return item_grid(a.nx, a.ny, a.nz); }
 inline ItemGrid pair_grid(const Args& a) { return item_grid(a.nx / 2, a.ny, a.nz); }
@@ -2679,7 +2688,7 @@ struct Impl {
                 return;
             }
         }
-        launch_after(k_step<P, KIND, FLOW, TAPE>, node_grid(a), start_early<P>(a), s, a, (const T*)fs, (T*)fd,
+        launch_after(k_step<P, KIND, FLOW, TAPE>, step_grid<P>(a), start_early<P>(a), s, a, (const T*)fs, (T*)fd,
                      (const TGp*)gs, (TGp*)gd, hp, (C*)tape_e, (C*)tape_m);
     }
     static void step(const Args& a, StepKind kind, const void* fs, void* fd, const void* gs,
