@@ -414,8 +414,11 @@ lbpc_status lbpc_step(lbpc_handle* h, int n) {
         if (rep > 0) take = (int)std::min<long long>(take, rep - h->step % rep);
         if (take < CLUSTER_LEAST) take = 1;
         if (take > 1) {
+            // the state ends in the buffer that single steps would leave it in, so that a
+            // captured call can be replayed (the launch reads all of its input before it
+            // writes, so that may be the one it came from)
             const bool aa = h->p.streaming == LBPC_AA;
-            const int nb = aa ? h->cur : 1 - h->cur;
+            const int nb = aa || take % 2 == 0 ? h->cur : 1 - h->cur;
             LBPC_CK(h, h->L->cluster_steps(h->args, aa, h->f[h->cur], h->f[nb], h->g[h->cur],
                                            h->g[nb], h->hp, take, (int)(h->step % 2), h->stream));
             h->cur = nb;

@@ -78,3 +78,31 @@ def test_blocks_of_steps_equal_single_steps(flow_model, precision, shapes, strea
             assert np.array_equal(a.history(), b.history()), (shape, bc)
             if streaming == inp.PULL:
                 assert a.save() == b.save(), (shape, bc)
+
+
+@pytest.mark.parametrize("shape,precision,flow_model,streaming", [
+    ((64, 16, 16), inp.FP32, inp.FLOW_MRT, inp.PULL), ((16, 8, 8), inp.FP32, inp.FLOW_MRT, inp.PULL),
+    ((64, 4, 4), inp.FP64, inp.FLOW_NONE, inp.PULL), ((24, 24, 24), inp.FP64, inp.FLOW_MRT, inp.PULL),
+    ((33, 16, 16), inp.FP16, inp.FLOW_MRT, inp.AA), ((16, 8, 8), inp.FP32, inp.FLOW_MRT, inp.AA)])
+def test_captured_steps_can_be_replayed(shape, precision, flow_model, streaming):
+    """An even number of steps recorded into a CUDA graph, replayed, equals the same calls."""
+    p = inp.Params(precision=precision, flow_model=flow_model, streaming=streaming, Ra=1e5, Pr=0.7,
+                   tau_g=0.0 if flow_model else 0.8, report_every=10 ** 6)
+    h0 = np.random.default_rng(0).uniform(-0.2, 1.5, int(np.prod(shape)))
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        a, b = LBPC(shape, p, stream=s), LBPC(shape, p, stream=s)
+        for v in (a, b):
+            v.set_initial_h(h0)
+            v.step(6)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            a.step(6)
+        for _ in range(3):
+            graph.replay()
+            b.step(6)
+        A, R = a.fields(), b.fields()
+        s.synchronize()
+        for k, v in A.items():
+            assert torch.equal(v, R[k]), k
