@@ -2722,10 +2722,13 @@ struct Impl {
                                  double* hp, int n, int odd, int* fits, cudaStream_t s) {
         auto* kern = k_steps_cluster<P, FLOW, AA>;
         const int per = (a.N + CL_CTAS - 1) / CL_CTAS;
-        const size_t bytes = 2 * (size_t)per * ((FLOW ? 19 * sizeof(T) : 0) + 6 * sizeof(TGp));
+        constexpr size_t node = 2 * ((FLOW ? 19 * sizeof(T) : 0) + 6 * sizeof(TGp));
+        const size_t bytes = per * node;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+            // the same limit whatever the handle: other threads may be launching this kernel
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(CL_THREADS<P, FLOW> * node));
         if (e != cudaSuccess) return e;
         cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension;
