@@ -1079,8 +1079,16 @@ LBPC_HD double excess_minus(double e, const typename Store<P>::C* g) {
 // ---------------------------------------------------------------------------------
 // Node-level operations (host + device: the kernels below call them once per node).
 // ---------------------------------------------------------------------------------
-// Largest lattice the pair paths take: they form plane offsets of up to 3 N in int.
-constexpr int kPairMaxN = 715827882;  // floor((2^31 - 1) / 3)
+// Whether the pair paths take a lattice: even nx, and element offsets that fit in an int.  They
+// form offsets from a population's plane: of a neighbour, below N; at a wall of the reflected
+// population at the node itself, whose plane lies up to three planes away (q = 7 and 10, 11
+// and 14), below 4 N.  (The plane distance alone, up to 3 N, is formed without walls too.)
+constexpr int kPairMaxN = 536870911;      // 4 N < 2^31
+constexpr int kPairMaxNOpen = 715827882;  // 3 N < 2^31
+LBPC_HD bool pairs_fit(const Args& a) {
+    const bool walls = a.wall[0] || a.wall[1] || a.wall[2] || a.wall[3] || a.wall[4] || a.wall[5];
+    return a.nx % 2 == 0 && a.N <= (walls ? kPairMaxN : kPairMaxNOpen);
+}
 
 template <int KIND> struct KindLayout;
 template <> struct KindLayout<STEP_PULL> { static constexpr int value = LAYOUT_PULL; };
@@ -1269,7 +1277,7 @@ LBPC_HD void gather_pair_pull(const Args& a, const NB& nb, int x0, int y, int z,
     using PRG = Pair<Mode<P>::G>;
     const Coef<C>& k = coef<C>(a);
     const size_t N = (size_t)a.N;
-    const int N32 = a.N;  // 3 N < 2^31 (kPairMaxN)
+    const int N32 = a.N;  // offsets in int: pairs_fit()
     const int n0 = x0 + a.nx * (y + a.ny * z), n1 = n0 + 1;
     const bool xlo = x0 == 0, xhi = x0 + 1 == a.nx - 1;
     const bool wlo = xlo && a.wall[0], whi = xhi && a.wall[1];
@@ -1298,7 +1306,7 @@ LBPC_HD void step_pair_pull(const Args& a, const NB& nb, int x0, int y, int z, c
     using PRG = Pair<Mode<P>::G>;
     const Coef<C>& k = coef<C>(a);
     const size_t N = (size_t)a.N;
-    const int N32 = a.N;  // 3 N < 2^31 (kPairMaxN)
+    const int N32 = a.N;  // offsets in int: pairs_fit()
     const int n0 = x0 + a.nx * (y + a.ny * z), n1 = n0 + 1;
     const bool xlo = x0 == 0, xhi = x0 + 1 == a.nx - 1;
     const bool wlo = xlo && a.wall[0], whi = xhi && a.wall[1];
@@ -1354,7 +1362,7 @@ LBPC_HD void step_pair_aa(const Args& a, int x0, int y, int z, TF<P>* F, TG<P>* 
     using PRG = Pair<Mode<P>::G>;
     const Coef<C>& k = coef<C>(a);
     const size_t N = (size_t)a.N;
-    const int N32 = a.N;  // 3 N < 2^31 (kPairMaxN)
+    const int N32 = a.N;  // offsets in int: pairs_fit()
     const int sy = a.nx, sz = a.nx * a.ny;
     const int n0 = x0 + a.nx * (y + a.ny * z), n1 = n0 + 1;
     const bool xlo = x0 == 0, xhi = x0 + 1 == a.nx - 1;
@@ -2049,7 +2057,7 @@ LBPC_HD CT<P> adj_reverse_pair(const Args& a, const NB& nb, int x0, int y, int z
     using VC = typename Vec2<C>::type;
     const Coef<C>& k = coef<C>(a);
     const size_t N = (size_t)a.N;
-    const int N32 = a.N;  // 3 N < 2^31 (kPairMaxN)
+    const int N32 = a.N;  // offsets in int: pairs_fit()
     constexpr int nf = FLOW ? 19 : 0;
     const int n0 = x0 + a.nx * (y + a.ny * z), n1 = n0 + 1;
     const bool xlo = x0 == 0, xhi = x0 + 1 == a.nx - 1;
@@ -2678,7 +2686,7 @@ struct Impl {
                        void* tape_m = nullptr) {
         using C = CT<P>;
         if constexpr (P != LBPC_FP64) {  // FP64 keeps one node per thread
-            if (a.nx % 2 == 0 && a.N <= kPairMaxN) {
+            if (pairs_fit(a)) {
                 if constexpr (KIND == STEP_PULL)
                     launch_after(k_step_pull_x2<P, FLOW, TAPE>, pair_grid(a), true, s, a, (const T*)fs,
                                  (T*)fd, (const TGp*)gs, (TGp*)gd, hp, (C*)tape_e, (C*)tape_m);
@@ -2787,7 +2795,7 @@ struct Impl {
     static void macro_k(const Args& a, const void* f, const void* g, const double* hp,
                         const MacroOut& o, cudaStream_t s) {
         if constexpr (P != LBPC_FP64 && LAYOUT == LAYOUT_PULL) {
-            bool pairs = a.nx % 2 == 0 && a.N <= kPairMaxN;
+            bool pairs = pairs_fit(a);
             for (double* v : {o.T, o.fl, o.h, o.rho, o.ux, o.uy, o.uz})
                 pairs = pairs && ((uintptr_t)v & 15) == 0;  // the caller's arrays
             if (pairs) {
@@ -2863,7 +2871,7 @@ struct Impl {
         using C = CT<P>;
         if constexpr (P != LBPC_FP64) {
             // the paired grid never has more warps than the per-node one that sized Lpart
-            if (a.nx % 2 == 0 && a.N <= kPairMaxN) {
+            if (pairs_fit(a)) {
                 launch_after(a.flow ? k_adj_reverse_x2<P, true> : k_adj_reverse_x2<P, false>,
                              pair_grid(a), true, s, a, (const C*)lin, (C*)lout, (const C*)tape_e,
                              (const C*)tape_m, wface, gtw, Lpart);
