@@ -601,61 +601,138 @@ LBPC_HD C solid_phi(const Coef<C>& k, C fl, C* dphi = nullptr) {
     return fl;
 }
 
-#if defined(__CUDA_ARCH__)
 // ---------------------------------------------------------------------------------
-// FP64 flow collision with its sums in 64-bit integers.
+// FP64 flow collision with its sums in integers.
 //
 // GB300 issues one FP64 warp instruction per 16 cycles and SM, whatever it is; of the 300 of a
 // step 230 were additions of the moment transforms.  Populations between 2^-6 and 2^-1 (every
 // state near the rest weights 1/3, 1/18, 1/36) are multiples of 2^-58, so their sums are exact
-// in integers of that unit, two instructions on the integer pipes each; so are the sums of the
-// back-transform in units of 2^-64, to which the corrections d_k are rounded.  What is left to
-// the FP64 pipe are the products.  The error is no larger than of FP64 sums: the moments are
-// exact instead of rounded at each addition, a correction is off by 2^-65 and enters times 30
-// at most (2^-60, against half an ulp of f, 2^-59 to 2^-55), and f* is rounded once.
-// Against quadruple precision, one step from half-melted states: 0.24 ulp rms and 0.6 at most,
-// where FP64 sums gave 0.65 to 0.93 and 4.3.
-// 128^3: 305 FP64 instructions per node and 1110 us a step before, 161 and 537 us now.
+// in 64-bit integers of that unit, two instructions on the integer pipes each; so are the sums
+// of the back-transform, in units of 2^-85, where a correction d_k keeps all of its bits down to
+// |d_k| = 2^-33 and is off by 2^-86 at most (half an ulp of f: 2^-59 to 2^-55).  What is left to
+// the FP64 pipe are the products.  The moments are exact and rounded once, so is f*, to nearest
+// even: its ties are not rare, and rounded up they would add 5e-19 to the mass of every node in
+// every step.
+// Against quadruple precision, one collision of states near rest: 0.29 ulp rms and 0.7 at most,
+// where FP64 sums give 0.93 to 0.98 and 4.3.
 // ---------------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long mantissa_of(unsigned hi, unsigned lo) {
-    return (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo;
+// (By 32-bit words and funnel shifts: a conversion is some twenty instructions, and 56 of them are
+// two thirds of a node's.)
+struct FxWords { unsigned hi, lo; };
+LBPC_HD FxWords fx_words(double v) {
+#if defined(__CUDA_ARCH__)
+    return {(unsigned)__double2hiint(v), (unsigned)__double2loint(v)};
+#else
+    unsigned long long u;
+    std::memcpy(&u, &v, 8);
+    return {(unsigned)(u >> 32), (unsigned)u};
+#endif
+}
+LBPC_HD double fx_make(unsigned hi, unsigned lo) {
+#if defined(__CUDA_ARCH__)
+    return __hiloint2double((int)hi, (int)lo);
+#else
+    const unsigned long long u = (unsigned long long)hi << 32 | lo;
+    double v;
+    std::memcpy(&v, &u, 8);
+    return v;
+#endif
+}
+// lower word of hi:lo >> s and upper word of hi:lo << s, s modulo 32
+LBPC_HD unsigned fx_shr(unsigned hi, unsigned lo, unsigned s) {
+#if defined(__CUDA_ARCH__)
+    return __funnelshift_r(lo, hi, s);
+#else
+    return (unsigned)(((unsigned long long)hi << 32 | lo) >> (s & 31u));
+#endif
+}
+LBPC_HD unsigned fx_shl(unsigned hi, unsigned lo, unsigned s) {
+#if defined(__CUDA_ARCH__)
+    return __funnelshift_l(lo, hi, s);
+#else
+    return (unsigned)(((unsigned long long)hi << 32 | lo) << (s & 31u) >> 32);
+#endif
+}
+LBPC_HD unsigned fx_clz(unsigned a) {  // 32 for zero
+#if defined(__CUDA_ARCH__)
+    return (unsigned)__clz((int)a);
+#else
+    return a ? (unsigned)__builtin_clz(a) : 32u;
+#endif
+}
+LBPC_HD unsigned long long fx_join(unsigned hi, unsigned lo) {
+    return (unsigned long long)hi << 32 | lo;
 }
 // f in units of 2^-58; ok: 2^-6 <= f < 2^-1
-__device__ __forceinline__ long long fx_load(double f, bool& ok) {
-    const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
-    ok &= hi - (1017u << 20) < (5u << 20);
-    return (long long)(mantissa_of(hi, lo) << (((hi >> 20) - 1017u) & 7u));
+LBPC_HD long long fx_load(double f, bool& ok) {
+    const FxWords w = fx_words(f);
+    ok &= w.hi - (1017u << 20) < (5u << 20);
+    const unsigned s = (w.hi >> 20) - 1017u, m = (w.hi & 0xfffffu) | 0x100000u;
+    return (long long)fx_join(fx_shl(m, w.lo, s), w.lo << (s & 31u));
 }
-// the double nearest to m 2^-unit (bits 10 and below of a 64-bit mantissa rounded half up)
-template <int UNIT>
-__device__ __forceinline__ unsigned long long fx_bits(unsigned long long a) {
-    const int n = __clzll((long long)a) & 63;
-    const unsigned long long m = a << n;
-    const unsigned long long b =
-        ((unsigned long long)(1085 - UNIT - n) << 52) + (m >> 11) + ((m >> 10) & 1ull);
-    return a ? b : 0ull;
+// x in units of 2^-58, to nearest (ties away from zero)
+LBPC_HD double fx_double(long long x) {
+    const unsigned long long s = (unsigned long long)(x >> 63);
+    const unsigned long long a = ((unsigned long long)x ^ s) - s;
+    unsigned hi = (unsigned)(a >> 32), lo = (unsigned)a, e = 1085u - 58u;
+    if (hi == 0) {
+        hi = lo;
+        lo = 0;
+        e -= 32u;
+    }
+    const unsigned n = fx_clz(hi);
+    hi = fx_shl(hi, lo, n);
+    lo <<= n & 31u;
+    unsigned long long b = fx_join((hi >> 11) + ((e - n) << 20), fx_shr(hi, lo, 11)) + ((lo >> 10) & 1u);
+    if (a == 0) b = 0;
+    return fx_make((unsigned)(b >> 32) | ((unsigned)s & 0x80000000u), (unsigned)b);
 }
-__device__ __forceinline__ double fx_double(long long x) {  // units of 2^-58
-    const long long s = x >> 63;
-    const unsigned long long b = fx_bits<58>((unsigned long long)((x ^ s) - s));
-    return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
+// A sum of corrections, (h + l 2^-24) 2^-61.  The parts are added by themselves: 24 bits in an int
+// leave room for the coefficients of the back-transform, so no carry runs between them.
+struct FxCorr {
+    unsigned long long h;
+    int l;
+};
+LBPC_HD FxCorr operator+(FxCorr a, FxCorr b) { return {a.h + b.h, a.l + b.l}; }
+LBPC_HD FxCorr operator-(FxCorr a, FxCorr b) { return {a.h - b.h, a.l - b.l}; }
+LBPC_HD FxCorr operator*(int k, FxCorr a) { return {(unsigned long long)(long long)k * a.h, k * a.l}; }
+// d, rounded to 2^-86; ok: |d| < 2^-4
+LBPC_HD FxCorr fx_corr(double d, bool& ok) {
+    const FxWords w = fx_words(d);
+    const unsigned ex = w.hi >> 20 & 0x7ffu;
+    ok &= ex <= 1018u;
+    // d = (u2:u1) 2^(ex - 1086), so u2:u1:u0 >> s has h in its upper two words
+    const unsigned s = 1025u - ex < 127u ? 1025u - ex : 127u;
+    unsigned u2 = fx_shl((w.hi & 0xfffffu) | 0x100000u, w.lo, 11), u1 = w.lo << 11, u0 = 0;
+    if (s & 32u) { u0 = u1; u1 = u2; u2 = 0; }
+    if (s & 64u) { u0 = u2; u1 = 0; u2 = 0; }
+    const unsigned long long h = fx_join(u2 >> (s & 31u), fx_shr(u2, u1, s));
+    const int l = (int)(((fx_shr(u1, u0, s) >> 7) + 1u) >> 1);
+    const int neg = (int)w.hi >> 31;
+    const unsigned long long neg2 = (unsigned long long)(long long)neg;
+    return {(h ^ neg2) - neg2, (l ^ neg) - neg};
 }
-// d in units of 2^-64, rounded half up; ok: |d| < 2^-7
-__device__ __forceinline__ long long fx_corr(double d, bool& ok) {
-    const int hi = __double2hiint(d), ex = hi >> 20 & 0x7ff;
-    ok &= ex <= 1015;
-    const unsigned long long m = mantissa_of((unsigned)hi, (unsigned)__double2loint(d)) << 8;
-    const int sh = 1018 - ex;
-    const long long r = (long long)(((m >> (sh < 63 ? sh : 63)) + 1ull) >> 1), s = hi >> 31;
-    return (r ^ s) - s;
+// f* = f + c, to nearest even; ok: f* >= 2^-7 (and its 53 bits then lie in the high part)
+LBPC_HD double fx_store(long long f, FxCorr c, bool& ok) {
+    const unsigned long long v = ((unsigned long long)f << 3) + c.h +
+                                 (unsigned long long)(long long)(c.l >> 24);
+    const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
+    ok &= (int)hi >= 1 << 22;
+    const unsigned n = fx_clz(hi), s = 11u - n;  // 2..8 bits below the 53
+    const unsigned q = fx_shr(hi, lo, s);
+    const unsigned rest = lo << ((n - 11u) & 31u) | ((unsigned)c.l & 0xffffffu);
+    const unsigned up = (unsigned)(((unsigned long long)rest + (0x7fffffffu + (q & 1u))) >> 32);
+    const unsigned long long b = fx_join((hi >> (s & 31u)) + ((1024u - n) << 20), q) + up;
+    return fx_make((unsigned)(b >> 32), (unsigned)b);
 }
-// f* = f + correction, units of 2^-64; ok: 0 < f* < 2^-1
-__device__ __forceinline__ double fx_store(long long f58, long long c64, bool& ok) {
-    const long long v = (f58 << 6) + c64;
-    ok &= v > 0;
-    return __longlong_as_double((long long)fx_bits<64>((unsigned long long)v));
+
+// All populations of a node in units of 2^-58; whether they lie in the range.
+LBPC_HD bool flow_fx_load(const double* f, long long* F) {
+    bool ok = true;
+#pragma unroll
+    for (int q = 0; q < 19; q++) F[q] = fx_load(f[q], ok);
+    return ok;
 }
-#endif
 
 template <class C>
 LBPC_HD void flow_sums(const C* f, const Coef<C>& k, C& rho, C& jx, C& jy, C& jz) {
@@ -673,23 +750,22 @@ template <class C>
 LBPC_HD void flow_macro(const C* f, const Coef<C>& k, C T, C fl, C& rho, C& jx,
                                            C& jy, C& jz, C& ux, C& uy, C& uz, C& Fx, C& Fy,
                                            C& Fz) {
-#if defined(__CUDA_ARCH__)
     if constexpr (sizeof(C) == 8) {  // integer sums (128^3: 283 us for the fields without)
-        bool ok = true;
         long long F[19];
+        if (flow_fx_load(f, F)) {
+            long long r = F[0];
 #pragma unroll
-        for (int q = 0; q < 19; q++) F[q] = fx_load(f[q], ok);
-        long long r = F[0];
-#pragma unroll
-        for (int q = 1; q < 19; q++) r += F[q];
-        rho = fx_double(r);
-        jx = fx_double((F[1] - F[2]) + (F[7] - F[8] + F[9] - F[10]) + (F[11] - F[12] + F[13] - F[14]));
-        jy = fx_double((F[3] - F[4]) + (F[7] + F[8] - F[9] - F[10]) + (F[15] - F[16] + F[17] - F[18]));
-        jz = fx_double((F[5] - F[6]) + (F[11] + F[12] - F[13] - F[14]) + (F[15] + F[16] - F[17] - F[18]));
-        if (!ok) flow_sums(f, k, rho, jx, jy, jz);
-    } else
-#endif
+            for (int q = 1; q < 19; q++) r += F[q];
+            rho = fx_double(r);
+            jx = fx_double((F[1] - F[2]) + (F[7] - F[8] + F[9] - F[10]) + (F[11] - F[12] + F[13] - F[14]));
+            jy = fx_double((F[3] - F[4]) + (F[7] + F[8] - F[9] - F[10]) + (F[15] - F[16] + F[17] - F[18]));
+            jz = fx_double((F[5] - F[6]) + (F[11] + F[12] - F[13] - F[14]) + (F[15] + F[16] - F[17] - F[18]));
+        } else {
+            flow_sums(f, k, rho, jx, jy, jz);
+        }
+    } else {
         flow_sums(f, k, rho, jx, jy, jz);
+    }
     const C Fb = k.gbeta * (T - k.Tref);
     const C usx = jx, usy = jy, usz = jz + C(0.5) * Fb;
     const C phi = solid_phi(k, fl);
@@ -867,20 +943,17 @@ LBPC_HD void collide_flow(C* f, const Coef<C>& k, C T, C fl, C& ux, C& uy, C& uz
     }
 }
 
-#if defined(__CUDA_ARCH__)
-// As collide_flow<false>; false (f is then not to be used) where a value lies outside the
-// ranges above.  No sum overflows within them: the moments stay below 9 x 2^58, the corrections'
-// sums below 42 x 2^57.
-__device__ __forceinline__ bool collide_flow_fx(double* f, const Coef<double>& k, double T,
-                                                double fl, double& ux, double& uy, double& uz,
-                                                double& rho_o, double& jx_o, double& jy_o,
-                                                double& jz_o) {
+// As collide_flow<false>, from populations that flow_fx_load accepted; false (f is then not to be
+// used) where a correction reaches 2^-4 or an f* falls below 2^-7.  No sum overflows: the
+// moments stay below 9 x 2^58; a sum of corrections, whose coefficients add up to 42 at most, stays
+// below 42 x 2^57 and in its low part at 42 x 2^24.
+LBPC_HD bool collide_flow_fx(const long long* F, double* f, const Coef<double>& k, double T,
+                             double fl, double& ux, double& uy, double& uz, double& rho_o,
+                             double& jx_o, double& jy_o, double& jz_o) {
     using C = double;
     using I = long long;
+    using W = FxCorr;
     bool ok = true;
-    I F[19];
-#pragma unroll
-    for (int q = 0; q < 19; q++) F[q] = fx_load(f[q], ok);
     const I a1 = F[1] + F[2], b1 = F[1] - F[2];
     const I a3 = F[3] + F[4], b3 = F[3] - F[4];
     const I a5 = F[5] + F[6], b5 = F[5] - F[6];
@@ -925,64 +998,82 @@ __device__ __forceinline__ bool collide_flow_fx(double* f, const Coef<double>& k
     const C pxx_eq = rho * (C(3) * uxx - u2), pww_eq = rho * (uyy - uzz);
     const C FFxx = C(6) * Fx * ux - C(2) * Fu, FFww = C(2) * (Fy * uy - Fz * uz);
     const C r23 = C(2.0 / 3.0) * rho;
-    const I d1 = fx_corr(k.r_e * (m1 - ru2) + k.c_e * Fu, ok);
-    const I d2 = fx_corr(k.r_eps * (m2 + C(5.5) * ru2) + k.c_eps * Fu, ok);
-    const I d3 = fx_corr(Fx * C(0.1), ok), d5 = fx_corr(Fy * C(0.1), ok),
-            d7 = fx_corr(Fz * C(0.1), ok);
-    const I d4 = fx_corr(k.r_q * (m4 + r23 * ux) + k.c_q * Fx, ok);
-    const I d6 = fx_corr(k.r_q * (m6 + r23 * uy) + k.c_q * Fy, ok);
-    const I d8 = fx_corr(k.r_q * (m8 + r23 * uz) + k.c_q * Fz, ok);
-    const I d9 = fx_corr(k.r_nu9 * (m9 - pxx_eq) + k.c_nu9 * FFxx, ok);
-    const I d10 = fx_corr(k.r_pi10 * (m10 + C(0.5) * pxx_eq) + k.c_pi10 * FFxx, ok);
-    const I d11 = fx_corr(k.r_nu11 * (m11 - pww_eq) + k.c_nu11 * FFww, ok);
-    const I d12 = fx_corr(k.r_pi12 * (m12 + C(0.5) * pww_eq) + k.c_pi12 * FFww, ok);
-    const I d13 = fx_corr(k.r_nu13 * (xy_p - rux * uy) + k.c_nu13 * (Fx * uy + Fy * ux), ok);
-    const I d14 = fx_corr(k.r_nu13 * (yz_p - rho * uy * uz) + k.c_nu13 * (Fy * uz + Fz * uy), ok);
-    const I d15 = fx_corr(k.r_nu13 * (xz_p - rux * uz) + k.c_nu13 * (Fx * uz + Fz * ux), ok);
-    const I d16 = fx_corr(k.r_t * m16, ok), d17 = fx_corr(k.r_t * m17, ok),
-            d18 = fx_corr(k.r_t * m18, ok);
+    const C d1 = k.r_e * (m1 - ru2) + k.c_e * Fu;
+    const C d2 = k.r_eps * (m2 + C(5.5) * ru2) + k.c_eps * Fu;
+    const C d3 = Fx * C(0.1), d5 = Fy * C(0.1), d7 = Fz * C(0.1);
+    const C d4 = k.r_q * (m4 + r23 * ux) + k.c_q * Fx;
+    const C d6 = k.r_q * (m6 + r23 * uy) + k.c_q * Fy;
+    const C d8 = k.r_q * (m8 + r23 * uz) + k.c_q * Fz;
+    const C d9 = k.r_nu9 * (m9 - pxx_eq) + k.c_nu9 * FFxx;
+    const C d10 = k.r_pi10 * (m10 + C(0.5) * pxx_eq) + k.c_pi10 * FFxx;
+    const C d11 = k.r_nu11 * (m11 - pww_eq) + k.c_nu11 * FFww;
+    const C d12 = k.r_pi12 * (m12 + C(0.5) * pww_eq) + k.c_pi12 * FFww;
+    const C d13 = k.r_nu13 * (xy_p - rux * uy) + k.c_nu13 * (Fx * uy + Fy * ux);
+    const C d14 = k.r_nu13 * (yz_p - rho * uy * uz) + k.c_nu13 * (Fy * uz + Fz * uy);
+    const C d15 = k.r_nu13 * (xz_p - rux * uz) + k.c_nu13 * (Fx * uz + Fz * ux);
+    const C d16 = k.r_t * m16, d17 = k.r_t * m17, d18 = k.r_t * m18;
 
-    // back-transform (columns of Eq. 51), sums shared as in collide_flow
-    const I eax = -11 * d1 - 4 * d2, edg = 8 * d1 + d2;
-    f[0] = fx_store(F[0], -30 * d1 + 12 * d2, ok);
-    const I ox = d3 - 4 * d4, oy = d5 - 4 * d6, oz = d7 - 4 * d8;
-    const I ex1 = eax + 2 * d9 - 4 * d10;
-    const I cyz = eax - d9 + 2 * d10, w11 = d11 - 2 * d12;
-    const I ey1 = cyz + w11, ez1 = cyz - w11;
-    f[1] = fx_store(F[1], ex1 + ox, ok);
-    f[2] = fx_store(F[2], ex1 - ox, ok);
-    f[3] = fx_store(F[3], ey1 + oy, ok);
-    f[4] = fx_store(F[4], ey1 - oy, ok);
-    f[5] = fx_store(F[5], ez1 + oz, ok);
-    f[6] = fx_store(F[6], ez1 - oz, ok);
-    const I X = d3 + d4, Y = d5 + d6, Z = d7 + d8;
-    const I a910 = edg + d9 + d10, b1112 = d11 + d12;
-    const I exy = a910 + b1112, exz = a910 - b1112;
-    const I eyz = edg - 2 * d9 - 2 * d10;
+    // back-transform (columns of Eq. 51), sums shared as in collide_flow; the odd corrections
+    // stay doubles (half the registers) until their sums
+    W ex1, ey1, ez1, exy, exz, eyz;
     {
-        const I u = X + d16, v = Y - d17, Pp = exy + d13, Qq = exy - d13;
-        f[7] = fx_store(F[7], Pp + (u + v), ok);
-        f[8] = fx_store(F[8], Qq + (v - u), ok);
-        f[9] = fx_store(F[9], Qq - (v - u), ok);
-        f[10] = fx_store(F[10], Pp - (u + v), ok);
+        const W w1 = fx_corr(d1, ok), w2 = fx_corr(d2, ok);
+        f[0] = fx_store(F[0], -30 * w1 + 12 * w2, ok);
+        const W w9 = fx_corr(d9, ok), w10 = fx_corr(d10, ok);
+        const W w11 = fx_corr(d11, ok), w12 = fx_corr(d12, ok);
+        const W eax = -11 * w1 - 4 * w2, edg = 8 * w1 + w2;
+        const W cyz = eax - w9 + 2 * w10, v11 = w11 - 2 * w12, a910 = w9 + w10, b1112 = w11 + w12;
+        ex1 = eax + 2 * w9 - 4 * w10;
+        ey1 = cyz + v11;
+        ez1 = cyz - v11;
+        exy = edg + a910 + b1112;
+        exz = edg + a910 - b1112;
+        eyz = edg - 2 * a910;
+    }
+    W X, Y, Z;
+    {
+        const W w3 = fx_corr(d3, ok), w4 = fx_corr(d4, ok), o = w3 - 4 * w4;
+        f[1] = fx_store(F[1], ex1 + o, ok);
+        f[2] = fx_store(F[2], ex1 - o, ok);
+        X = w3 + w4;
     }
     {
-        const I u = X - d16, v = Z + d18, Pp = exz + d15, Qq = exz - d15;
-        f[11] = fx_store(F[11], Pp + (u + v), ok);
-        f[12] = fx_store(F[12], Qq + (v - u), ok);
-        f[13] = fx_store(F[13], Qq - (v - u), ok);
-        f[14] = fx_store(F[14], Pp - (u + v), ok);
+        const W w5 = fx_corr(d5, ok), w6 = fx_corr(d6, ok), o = w5 - 4 * w6;
+        f[3] = fx_store(F[3], ey1 + o, ok);
+        f[4] = fx_store(F[4], ey1 - o, ok);
+        Y = w5 + w6;
     }
     {
-        const I u = Y + d17, v = Z - d18, Pp = eyz + d14, Qq = eyz - d14;
-        f[15] = fx_store(F[15], Pp + (u + v), ok);
-        f[16] = fx_store(F[16], Qq + (v - u), ok);
-        f[17] = fx_store(F[17], Qq - (v - u), ok);
-        f[18] = fx_store(F[18], Pp - (u + v), ok);
+        const W w7 = fx_corr(d7, ok), w8 = fx_corr(d8, ok), o = w7 - 4 * w8;
+        f[5] = fx_store(F[5], ez1 + o, ok);
+        f[6] = fx_store(F[6], ez1 - o, ok);
+        Z = w7 + w8;
+    }
+    const W w16 = fx_corr(d16, ok), w17 = fx_corr(d17, ok);
+    {
+        const W u = X + w16, v = Y - w17, w = fx_corr(d13, ok), p = exy + w, m = exy - w;
+        f[7] = fx_store(F[7], p + (u + v), ok);
+        f[8] = fx_store(F[8], m + (v - u), ok);
+        f[9] = fx_store(F[9], m - (v - u), ok);
+        f[10] = fx_store(F[10], p - (u + v), ok);
+    }
+    const W w18 = fx_corr(d18, ok);
+    {
+        const W u = X - w16, v = Z + w18, w = fx_corr(d15, ok), p = exz + w, m = exz - w;
+        f[11] = fx_store(F[11], p + (u + v), ok);
+        f[12] = fx_store(F[12], m + (v - u), ok);
+        f[13] = fx_store(F[13], m - (v - u), ok);
+        f[14] = fx_store(F[14], p - (u + v), ok);
+    }
+    {
+        const W u = Y + w17, v = Z - w18, w = fx_corr(d14, ok), p = eyz + w, m = eyz - w;
+        f[15] = fx_store(F[15], p + (u + v), ok);
+        f[16] = fx_store(F[16], m + (v - u), ok);
+        f[17] = fx_store(F[17], m - (v - u), ok);
+        f[18] = fx_store(F[18], p - (u + v), ok);
     }
     return ok;
 }
-#endif
 
 // D3Q7 enthalpy collision on the six moving populations (Eq. 21-25; SRT when every
 // rate equals 1/tau_g).  With d_a = g_a - g_a^eq, d_0 = -sum d_a (h is conserved), the
@@ -1101,12 +1192,10 @@ template <> struct KindLayout<STEP_AA_ODD> { static constexpr int value = LAYOUT
 // form there costs the pair path 1-5% in spills).
 // FX: FP64 flow collides with integer sums; a node outside their ranges (found before anything
 // is stored) is done again with FP64 sums.
-#if defined(__CUDACC__)
 template <int P, int KIND, int FLOW, bool TAPE>
-__device__ __noinline__ void step_node_fp64(const Args& a, int x, int y, int z, const TF<P>* fs,
-                                            TF<P>* fd, const TG<P>* gs, TG<P>* gd, double* hp,
-                                            CT<P>* tape_e, CT<P>* tape_m);
-#endif
+LBPC_HD_CALL void step_node_fp64(const Args& a, int x, int y, int z, const TF<P>* fs, TF<P>* fd,
+                                 const TG<P>* gs, TG<P>* gd, double* hp, CT<P>* tape_e,
+                                 CT<P>* tape_m);
 template <int P, int KIND, int FLOW, bool TAPE = false, bool FACE = false, bool FX = P == LBPC_FP64>
 LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
                        TF<P>* fd, const TG<P>* gs,
@@ -1136,15 +1225,16 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     C ux = C(0), uy = C(0), uz = C(0), rho = C(0), jx = C(0), jy = C(0), jz = C(0);
     if constexpr (FLOW) {  // FLOW 2: the drag closure, phi(f_l) in place of f_l
         const C phi = FLOW == 2 ? darcy_phi(k, fl) : fl;
-#if defined(__CUDA_ARCH__)
         if constexpr (FX) {
-            if (!collide_flow_fx(f, k, T, phi, ux, uy, uz, rho, jx, jy, jz)) {
+            long long F[19];
+            if (!flow_fx_load(f, F) ||
+                !collide_flow_fx(F, f, k, T, phi, ux, uy, uz, rho, jx, jy, jz)) {
                 step_node_fp64<P, KIND, FLOW, TAPE>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
                 return;
             }
-        } else
-#endif
+        } else {
             collide_flow<kRebuild<P>>(f, k, T, phi, ux, uy, uz, rho, jx, jy, jz);
+        }
     }
     if constexpr (TAPE) {  // macroscopic tape of the pre-collision state (adjoint)
         tape_e[n] = tape_excess(a, e, C(0));
@@ -1165,14 +1255,12 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     }
     hp[n] = excess_minus<Mode<P>::G>(e, g);
 }
-#if defined(__CUDACC__)
 template <int P, int KIND, int FLOW, bool TAPE>
-__device__ __noinline__ void step_node_fp64(const Args& a, int x, int y, int z, const TF<P>* fs,
-                                            TF<P>* fd, const TG<P>* gs, TG<P>* gd, double* hp,
-                                            CT<P>* tape_e, CT<P>* tape_m) {
+LBPC_HD_CALL void step_node_fp64(const Args& a, int x, int y, int z, const TF<P>* fs, TF<P>* fd,
+                                 const TG<P>* gs, TG<P>* gd, double* hp, CT<P>* tape_e,
+                                 CT<P>* tape_m) {
     step_node<P, KIND, FLOW, TAPE, false, false>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
 }
-#endif
 
 // Inversion and both collisions of a node pair (n0, n0 + 1), in registers; with TAPE also
 // the macroscopic tape of the pair's pre-collision state (adjoint).

@@ -6,6 +6,11 @@
 #include "lbpc_internal.h"
 
 #define LBPC_HD __host__ __device__ __forceinline__
+#if defined(__CUDACC__)
+#define LBPC_HD_CALL __host__ __device__ __noinline__  // kept out of its caller's registers
+#else
+#define LBPC_HD_CALL inline
+#endif
 
 namespace lbpc {
 
