@@ -726,12 +726,17 @@ LBPC_HD double fx_store(long long f, FxCorr c, bool& ok) {
     return fx_make((unsigned)(b >> 32), (unsigned)b);
 }
 
-// All populations of a node in units of 2^-58; whether they lie in the range.
+// All populations of a node in units of 2^-58; whether they lie in the range and sum up to less
+// than 4 (so that no moment overflows, see collide_flow_fx).
 LBPC_HD bool flow_fx_load(const double* f, long long* F) {
     bool ok = true;
+    unsigned long long rho = 0;
 #pragma unroll
-    for (int q = 0; q < 19; q++) F[q] = fx_load(f[q], ok);
-    return ok;
+    for (int q = 0; q < 19; q++) {
+        F[q] = fx_load(f[q], ok);
+        rho += (unsigned long long)F[q];
+    }
+    return ok && rho < 1ull << 60;
 }
 
 template <class C>
@@ -944,9 +949,10 @@ LBPC_HD void collide_flow(C* f, const Coef<C>& k, C T, C fl, C& ux, C& uy, C& uz
 }
 
 // As collide_flow<false>, from populations that flow_fx_load accepted; false (f is then not to be
-// used) where a correction reaches 2^-4 or an f* falls below 2^-7.  No sum overflows: the
-// moments stay below 9 x 2^58; a sum of corrections, whose coefficients add up to 42 at most, stays
-// below 42 x 2^57 and in its low part at 42 x 2^24.
+// used) where a correction reaches 2^-4 or an f* falls below 2^-7.  No sum overflows: the F are
+// positive with a sum below 2^60 and F_0 < 2^57, so a moment, whose coefficients are 7 at most but
+// for the 9 of F_0, stays below 7 x 2^60; a sum of corrections, whose coefficients add up to 42 at
+// most, stays below 42 x 2^57 and in its low part at 42 x 2^24.
 LBPC_HD bool collide_flow_fx(const long long* F, double* f, const Coef<double>& k, double T,
                              double fl, double& ux, double& uy, double& uz, double& rho_o,
                              double& jx_o, double& jy_o, double& jz_o) {

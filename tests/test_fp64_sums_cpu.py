@@ -4,6 +4,7 @@
   conversions give (to nearest even), and fx_corr keeps every bit of a correction down to 2^-33.
 * One collision against quadruple precision, over states near the rest weights with a share of
   solid and mushy nodes: errors in ulps of f* no larger than those of FP64 sums.
+* The largest moments that populations in range can have do not overflow 64 bits.
 * Mass of a periodic box with buoyancy and melting: rounding to nearest changes the sum of the
   populations of a node by 0.29 ulp rms each, 2^-54 for f_0 and less for the others, in either
   direction, so steps over N nodes move the mean by 0.29 x 2^-54 sqrt(steps / N).
@@ -36,12 +37,12 @@ static const double w[19] = {1. / 3, 1. / 18, 1. / 18, 1. / 18, 1. / 18, 1. / 18
                              1. / 36, 1. / 36, 1. / 36, 1. / 36, 1. / 36, 1. / 36,
                              1. / 36, 1. / 36, 1. / 36, 1. / 36, 1. / 36, 1. / 36};
 static Args a;
-static void setup(int n, double Pr, int wall, double s_eps) {
+static void setup(int n, double Pr, int wall, double rate) {
     lbpc_params p;
     std::memset(&p, 0, sizeof p);
     p.flow_model = LBPC_FLOW_MRT; p.enth_model = LBPC_ENTH_MRT; p.precision = LBPC_FP64;
     for (int f = 0; f < 6; f++) p.bc[f] = wall;
-    p.Ra = 1e5; p.Pr = Pr; p.St = 0.5; p.Ma = 0.1; p.s_eps = s_eps;
+    p.Ra = 1e5; p.Pr = Pr; p.St = 0.5; p.Ma = 0.1; p.s_e = p.s_eps = rate;
     p.Th = 1; p.Tref = 0.3; p.Cp_s = p.Cp_l = p.Cp_ref = 1; p.omega_T = 0.25; p.h0 = -1;
     Derived d; std::string e;
     if (!validate_and_map(n, n, n, &p, d, e)) { puts(e.c_str()); exit(2); }
@@ -146,9 +147,30 @@ static void drift(int n, int steps) {
                                                  g[s & 1].data(), g[1 - (s & 1)].data(), hp.data())));
     printf("%g\n", (double)((mass(f[steps & 1]) - before) / N));
 }
+// moving populations at the upper bound, f_0 small: m2 = 9 f_0 - 7 sum f_1..6 - 2 sum f_7..18 is
+// near -33; low relaxation rates, so that the correction stays in range whatever the moment is
+static void largest_moments() {
+    setup(32, 0.7, LBPC_ADIABATIC, 0.01);
+    const Coef<Quad> kq = quad(a.cd);
+    double worst = 0;
+    for (double f0 = 0x1p-6; f0 < 0.5; f0 += 0x1p-8)
+        for (double top : {std::nextafter(0.5, 0.0), 0.45, 0.3, 0.2}) {
+            double f[19], u[3], m[4];
+            Quad r[19], uq[3], mq[4];
+            long long F[19];
+            for (int q = 0; q < 19; q++) r[q] = f[q] = q ? top : f0;
+            if (!flow_fx_load(f, F) || !collide_flow_fx(F, f, a.cd, 0.3, 1.0, u[0], u[1], u[2], m[0],
+                                                        m[1], m[2], m[3]))
+                continue;  // FP64 sums take it
+            collide_flow<false>(r, kq, (Quad)0.3, (Quad)1, uq[0], uq[1], uq[2], mq[0], mq[1], mq[2], mq[3]);
+            for (int q = 0; q < 19; q++) worst = std::fmax(worst, std::fabs((double)((Quad)f[q] - r[q])));
+        }
+    printf("%g\n", worst);
+}
 int main(int argc, char** argv) {
     if (argv[1][0] == 'c') return conversions();
     if (argv[1][0] == 'e') errors(atof(argv[2]));
+    if (argv[1][0] == 'm') largest_moments();
     if (argv[1][0] == 'd') drift(atoi(argv[2]), atoi(argv[3]));
     return 0;
 }
@@ -187,6 +209,11 @@ def test_error_of_a_collision_is_no_larger_than_with_fp64_sums(harness, Pr):
     assert rms <= rms64 and largest <= largest64
     # half an ulp from the store, the rest from the products of the corrections
     assert rms <= 0.35 and largest <= 1.0
+
+
+def test_moments_do_not_overflow(harness):
+    # populations below 1, moments up to 33: a few roundings of f* and of the corrections
+    assert harness("moments")[0] <= 4 * 2.0 ** -53
 
 
 def test_mass_does_not_drift(harness):
