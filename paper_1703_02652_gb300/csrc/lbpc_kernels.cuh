@@ -604,8 +604,8 @@ LBPC_HD C solid_phi(const Coef<C>& k, C fl, C* dphi = nullptr) {
 // ---------------------------------------------------------------------------------
 // FP64 flow collision with its sums in integers.
 //
-// GB300 issues one FP64 warp instruction per 16 cycles and SM, whatever it is; of the 300 of a
-// step 230 were additions of the moment transforms.  Populations between 2^-6 and 2^-1 (every
+// GB300 issues one FP64 warp instruction per 16 cycles and SM, whatever it is; most of the 315 of
+// a step with FP64 sums are additions of the moment transforms.  Populations between 2^-6 and 2^-1 (every
 // state near the rest weights 1/3, 1/18, 1/36) are multiples of 2^-58, so their sums are exact
 // in 64-bit integers of that unit, two instructions on the integer pipes each; so are the sums
 // of the back-transform, in units of 2^-85, where a correction d_k keeps all of its bits down to
@@ -614,7 +614,8 @@ LBPC_HD C solid_phi(const Coef<C>& k, C fl, C* dphi = nullptr) {
 // even: its ties are not rare, and rounded up they would add 5e-19 to the mass of every node in
 // every step.
 // Against quadruple precision, one collision of states near rest: 0.29 ulp rms and 0.7 at most,
-// where FP64 sums give 0.93 to 0.98 and 4.3.
+// where FP64 sums give 0.93 to 0.98 and 4.3.  64^3 cavity: 131 FP64 instructions a warp and step
+// of 2870 in all, 79% of the FP64 pipe busy (FP64 sums: 315 of 2180); 128^3: 537 us a step.
 // ---------------------------------------------------------------------------------
 // (By 32-bit words and funnel shifts: a conversion is some twenty instructions, and 56 of them are
 // two thirds of a node's.)
@@ -1187,6 +1188,14 @@ LBPC_HD bool pairs_fit(const Args& a) {
     return a.nx % 2 == 0 && a.N <= (walls ? kPairMaxN : kPairMaxNOpen);
 }
 
+LBPC_HD bool warp_all(bool v) {
+#if defined(__CUDA_ARCH__)
+    return __all_sync(0xffffffffu, v);
+#else
+    return v;
+#endif
+}
+
 template <int KIND> struct KindLayout;
 template <> struct KindLayout<STEP_PULL> { static constexpr int value = LAYOUT_PULL; };
 template <> struct KindLayout<STEP_AA_EVEN> { static constexpr int value = LAYOUT_AA_NATURAL; };
@@ -1196,8 +1205,11 @@ template <> struct KindLayout<STEP_AA_ODD> { static constexpr int value = LAYOUT
 // flow collision, enthalpy collision, scatter, FP64 rest channel update.  FACE: for the rows
 // that the AA pair kernels leave to it, with the branch on the node's own position (the row
 // form there costs the pair path 1-5% in spills).
-// FX: FP64 flow collides with integer sums; a node outside their ranges (found before anything
-// is stored) is done again with FP64 sums.
+// FX: FP64 flow collides with integer sums.  Where a population lies outside their range, FP64
+// sums take the whole warp (128^3 with one fast column of nodes in each warp: 1083 us a step;
+// chosen by lanes, so that such a warp runs both forms, 1591; without a fast node 537).  A result
+// that leaves the range (found before anything is stored) sends its own node to FP64 sums.  All
+// lanes of the warp call this together then, those without a node with valid = false.
 template <int P, int KIND, int FLOW, bool TAPE>
 LBPC_HD_CALL void step_node_fp64(const Args& a, int x, int y, int z, const TF<P>* fs, TF<P>* fd,
                                  const TG<P>* gs, TG<P>* gd, double* hp, CT<P>* tape_e,
@@ -1206,7 +1218,7 @@ template <int P, int KIND, int FLOW, bool TAPE = false, bool FACE = false, bool 
 LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
                        TF<P>* fd, const TG<P>* gs,
                        TG<P>* gd, double* hp, CT<P>* tape_e = nullptr,
-                       CT<P>* tape_m = nullptr) {
+                       CT<P>* tape_m = nullptr, bool valid = true) {
     using C = CT<P>;
     const Coef<C>& k = coef<C>(a);
     const int n = x + a.nx * (y + a.ny * z);
@@ -1217,12 +1229,23 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     const Nb b = make_nb(a, x, y, z);
 
     C f[19], g[7];
-    if (inner) {
+    if (!valid) {
+        // (nothing to gather)
+    } else if (inner) {
         if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, HINT>(a, bi, n, fs, f);
         gather_g<Mode<P>::G, LAYOUT, HINT>(a, bi, n, x, y, z, gs, g);
     } else {
         if constexpr (FLOW) gather_f<Mode<P>::F, LAYOUT, HINT>(a, b, n, fs, f);
         gather_g<Mode<P>::G, LAYOUT, HINT>(a, b, n, x, y, z, gs, g);
+    }
+    long long F[FX && FLOW ? 19 : 1];
+    if constexpr (FX && FLOW) {
+        const bool in = warp_all(!valid || flow_fx_load(f, F));
+        if (!valid) return;
+        if (!in) {
+            step_node_fp64<P, KIND, FLOW, TAPE>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
+            return;
+        }
     }
     const double e = excess_plus<Mode<P>::G>(hp[n], g);  // h - h_s
 
@@ -1232,9 +1255,7 @@ LBPC_HD void step_node(const Args& a, int x, int y, int z, const TF<P>* fs,
     if constexpr (FLOW) {  // FLOW 2: the drag closure, phi(f_l) in place of f_l
         const C phi = FLOW == 2 ? darcy_phi(k, fl) : fl;
         if constexpr (FX) {
-            long long F[19];
-            if (!flow_fx_load(f, F) ||
-                !collide_flow_fx(F, f, k, T, phi, ux, uy, uz, rho, jx, jy, jz)) {
+            if (!collide_flow_fx(F, f, k, T, phi, ux, uy, uz, rho, jx, jy, jz)) {
                 step_node_fp64<P, KIND, FLOW, TAPE>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
                 return;
             }
@@ -2285,8 +2306,8 @@ k_step(const __grid_constant__ Args a, const TF<P>* fs, TF<P>* fd,
     int x, y, z;
     const bool valid = item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z);
     after_previous_grid(fs, fd, gs, gd, hp);
-    if (!valid) return;
-    step_node<P, KIND, FLOW, TAPE>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m);
+    if ((P != LBPC_FP64 || !FLOW) && !valid) return;
+    step_node<P, KIND, FLOW, TAPE>(a, x, y, z, fs, fd, gs, gd, hp, tape_e, tape_m, valid);
 }
 
 
