@@ -107,7 +107,7 @@ __global__ void k_fill(double* p, double v, int n) {
 __global__ void __launch_bounds__(256)
 k_finalize(const double* __restrict__ partial, const double* __restrict__ lines, int nx,
            double area, double nu_scale, double fd_scale, double step, int flow, int iso0,
-           double* __restrict__ result, double* __restrict__ hist_row) {
+           double* result, double* hist_row) {
     after_previous_grid(partial, lines);
     __shared__ double sh[256][NRED];
     double acc[NRED] = {0, 0, 0, 0, 0, 0};

@@ -2301,8 +2301,7 @@ constexpr int kNodeBlocks = !FLOW ? 1 : (P == LBPC_FP64 ? 3 : 8);
 template <int P, int KIND, int FLOW, bool TAPE>
 __global__ void __launch_bounds__(STEP_THREADS, kNodeBlocks<P, FLOW>)
 k_step(const __grid_constant__ Args a, const TF<P>* fs, TF<P>* fd,
-       const TG<P>* gs, TG<P>* gd, double* __restrict__ hp, CT<P>* __restrict__ tape_e,
-       CT<P>* __restrict__ tape_m) {
+       const TG<P>* gs, TG<P>* gd, double* hp, CT<P>* tape_e, CT<P>* tape_m) {
     int x, y, z;
     const bool valid = item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z);
     after_previous_grid(fs, fd, gs, gd, hp);
@@ -2323,8 +2322,7 @@ template <int P, int FLOW, bool TAPE>
 __global__ void __launch_bounds__(STEP_THREADS, TAPE ? (kRebuild<P> ? 5 : 4) : kPullBlocks<P>)
 k_step_pull_x2(const __grid_constant__ Args a, const TF<P>* fs,
                TF<P>* fd, const TG<P>* gs, TG<P>* gd,
-               double* __restrict__ hp, CT<P>* __restrict__ tape_e,
-               CT<P>* __restrict__ tape_m) {
+               double* hp, CT<P>* tape_e, CT<P>* tape_m) {
     int x0, y, z;
     const bool valid = item_cyz(a, a.nx / 2, a.by_hx, a.fill_hx, x0, y, z);
     x0 *= 2;
@@ -2360,7 +2358,7 @@ __device__ __noinline__ void aa_face_pair_call(const Args& a, int x0, int y, int
 // with 16-bit f and g six (80 registers; the odd step spills at six).
 template <int P, int FLOW, bool ODD>
 __global__ void __launch_bounds__(STEP_THREADS, sizeof(TG<P>) == 2 && !ODD ? 6 : 5)
-k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* __restrict__ hp) {
+k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* hp) {
     constexpr bool MIXED = kRebuild<P> && sizeof(TG<P>) == 4;
     int x0, y, z;
     const bool valid = item_cyz(a, a.nx / 2, a.by_hx, a.fill_hx, x0, y, z);
@@ -2715,9 +2713,9 @@ k_adj_seed(const __grid_constant__ Args a, const TG<P>* __restrict__ gs,
 template <int P, bool FLOW>
 __global__ void __launch_bounds__(STEP_THREADS)
 k_adj_reverse(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
-              CT<P>* __restrict__ lout, const CT<P>* __restrict__ tape_e,
+              CT<P>* lout, const CT<P>* __restrict__ tape_e,
               const CT<P>* __restrict__ tape_m, int wface, double* gtw,
-              double* __restrict__ Lpart) {
+              double* Lpart) {
     int x, y, z;
     CT<P> dL = CT<P>(0);
     const bool valid = item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z);
@@ -2741,9 +2739,9 @@ k_adj_reverse(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
 template <int P, bool FLOW>
 __global__ void __launch_bounds__(STEP_THREADS, 5)
 k_adj_reverse_x2(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
-                 CT<P>* __restrict__ lout, const CT<P>* __restrict__ tape_e,
+                 CT<P>* lout, const CT<P>* __restrict__ tape_e,
                  const CT<P>* __restrict__ tape_m, int wface, double* gtw,
-                 double* __restrict__ Lpart) {
+                 double* Lpart) {
     int x0, y, z;
     const bool valid = item_cyz(a, a.nx / 2, a.by_hx, a.fill_hx, x0, y, z);
     x0 *= 2;

@@ -31,10 +31,10 @@ LBPC_HD void opaque(T& v) {
 // In the kernels that follow one another on a stream, before any access to their data: lets
 // the next grid of the stream become resident while this one drains, then waits until the
 // previous grid has completed and its stores are visible.  The pointers given go through the
-// barrier: for data that the kernel only reads (const __restrict__) so that no load of it,
-// which the compiler may take for a constant, is moved above; in the pair kernels because the
-// compiler then forms addresses from them after it (which ones is a measurement: up to 8% of a
-// 16-bit step either way).
+// barrier.  A __restrict__ pointer has to: the compiler may take it that nothing else, the
+// barrier included, touches its data, and move a load above.  Others are held by the memory
+// clobber; those that the pair kernels pass all the same are a measurement (addresses are then
+// formed after the barrier: up to 8% of a 16-bit step either way).
 // Why: between two dependent launches the GPU waits in steps of about 2 us; 64^3 FP32 took
 // 10.3 us a step without the overlap and 8.0 us with it (6.2 -> 3.1 us at 64 x 1 x 64).
 template <class... Ptr>
