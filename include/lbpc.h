@@ -186,9 +186,11 @@ lbpc_status lbpc_set_wall_temperature(lbpc_handle *h, int face, const double *T_
 /* Advance n >= 0 time steps on the handle's stream.  Passages: one step is the pull
  * form of Eq. 5 (enthalpy, collision Eq. 6 SRT or Eq. 21-25 MRT with Eq. 47) and of Eq.
  * 50 (flow, collision Eq. 49 with Eq. 51-54), coupled through Eq. 2, Eq. 55 and Eq. 56,
- * with the walls of Sec. 3.1-3.3.  Lattices of up to 8192 nodes (FP32, 16-bit storage without
- * flow; 4096 in FP64 without flow) take four or more steps in one launch, with the bits of
- * the same steps one by one.  Divergence checks: with report_every > 0 the call is
+ * with the walls of Sec. 3.1-3.3.  Small lattices may take four or more steps in one launch,
+ * with the bits of the same steps one by one: up to 8192 nodes in FP32 (without the drag
+ * closure) and, without flow, in 16-bit storage, up to 4096 nodes in FP64 without flow, on a
+ * device that holds a cluster of 16 blocks; a launch ends at a diagnostics point and after
+ * 2048 steps.  Divergence checks: with report_every > 0 the call is
  * asynchronous unless it passes a diagnostics point; then it waits for the stream and
  * returns LBPC_ERR_DIVERGED if the last diagnostics it recorded saw a non-finite h or rho.
  * With report_every = 0 every call with n > 0 ends with one read of the stored g
