@@ -2294,8 +2294,11 @@ __device__ __forceinline__ bool item_cyz(const Args& a, int cols, const FastDiv&
     if (!item_cyz(a, a.nx, a.by_nx, a.fill_nx, x, y, z)) return;
 
 // One node per thread; with TAPE (pull) also the adjoint tape.
-// Blocks per SM: eight with 32- or 16-bit storage and flow (64 registers): 161 x 161 x 81 FP32
-// 83 us a step, 87 at seven, 92 at nine; FP64 flow three: 128^3 537 us, 591 at two.
+// Blocks per SM: eight with 32- or 16-bit storage and flow (64 registers; up to 72 bytes of spills
+// in the odd AA step).  161 x 161 x 81, us a step at eight and without a limit: FP32 82.9 and 85.9
+// (nine blocks 92), drag 85.4 and 93.1, AA 81.6 and 85.7, AA drag 81.6 and 87.0; FP16 60.5 and 64.4, AA
+// 61.3 and 66.2; FP16 with FP32 g 70.0 and 74.2, AA 71.1 and 77.8; BF16 as FP16.  FP64 flow three:
+// 128^3 537 us, 600 at two.
 template <int P, int FLOW>
 constexpr int kNodeBlocks = !FLOW ? 1 : (P == LBPC_FP64 ? 3 : 8);
 template <int P, int KIND, int FLOW, bool TAPE>
@@ -2766,22 +2769,27 @@ k_adj_reverse_x2(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
 // Host launchers.
 // ---------------------------------------------------------------------------------
 // FP64 lattices.  Grids of some warps per SM start after the one before instead: early blocks go
-// where that one left room, several to an SM beside idle ones, and share its FP64 pipe.  Blocks
-// of one warp spread best until there are many per SM.  us a step, early / after with 32 threads
-// a block, the better of the two with 128:
-//   flow, nodes       4096: 9.0 / 10.3, 9.3    8192: 13.3 / 10.3, 10.4   24,576: 18.1 / 13.1, 15.9
-//                   49,152: 18.7 / 18.6, 18.7   65,536: 23.8 / 26.7, 24.0  262,144: 74 / 76, 73
-//   conduction       8192: 3.7 / 6.2, 4.1    16,384: 4.6 / 6.2, 5.4    24,576: 11.5 / 6.3, 7.8
-//                   98,735: 15.5 / 14.4, 14.4  262,144: 25.2 / 26.7, 25.4
+// where that one left room, several to an SM beside idle ones, and share its FP64 pipe.  Up to
+// about one warp per scheduler (conduction) or per SM (flow) there is nothing to share, and large
+// grids fill every SM whenever they start.  Blocks of one warp spread best until there are many
+// per SM.  us a step, early / after with 32 threads a block, and the better of the two with 128
+// (cubes and n x 1 x n planes agree within 10%):
+//   flow         4624: 8.9 / 10.4, 8.8     6498: 9.0 / 10.3, 8.8      7200: 10.6 / 10.3, 8.7
+//                8000: 9.2 / 10.3, 10.3    9000: 13.0 / 10.3, 10.3   32,768: 17.5 / 14.4, 14.4
+//              46,656: 18.1 / 17.8, 18.1  49,152: 18.0 / 18.5, 18.0  57,798: 18.5 / 20.6, 18.4
+//             175,616: 50.9 / 53.4, 52.9 262,144: 73.2 / 75.8, 72.8
+//   conduction 13,824: 4.4 / 6.2, 5.4     19,200: 4.8 / 6.2, 4.7     20,480: 7.9 / 6.2, 6.1
+//              64,000: 12.9 / 10.3, 10.3 122,500: 15.5 / 14.6, 16.5 128,000: 16.2 / 16.5, 16.5
+//             216,000: 21.5 / 24.1, 22.1 238,328: 23.4 / 25.6, 23.8 262,144: 27.0 / 28.8, 27.1
 template <int P>
 inline bool start_early(const Args& a) {
     if (P != LBPC_FP64) return true;
-    return a.flow ? a.N <= 32 * SM_COUNT || a.N >= 3 * STEP_THREADS * SM_COUNT
-                  : a.N <= 112 * SM_COUNT || a.N >= 12 * STEP_THREADS * SM_COUNT;
+    return a.flow ? a.N <= 43 * SM_COUNT || a.N >= 320 * SM_COUNT
+                  : a.N <= 128 * SM_COUNT || a.N >= 832 * SM_COUNT;
 }
 template <int P>
 inline ItemGrid step_grid(const Args& a) {
-    const bool one_warp = P == LBPC_FP64 && a.N < 7 * STEP_THREADS * SM_COUNT;
+    const bool one_warp = P == LBPC_FP64 && a.N < 12 * STEP_THREADS * SM_COUNT;
     return item_grid(a.nx, a.ny, a.nz, one_warp ? 32 : STEP_THREADS);
 }
 inline ItemGrid node_grid(const Args& a) { return item_grid(a.nx, a.ny, a.nz); }
