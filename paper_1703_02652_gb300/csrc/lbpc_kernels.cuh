@@ -2781,11 +2781,16 @@ k_adj_reverse_x2(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
 //   conduction 13,824: 4.4 / 6.2, 5.4     19,200: 4.8 / 6.2, 4.7     20,480: 7.9 / 6.2, 6.1
 //              64,000: 12.9 / 10.3, 10.3 122,500: 15.5 / 14.6, 16.5 128,000: 16.2 / 16.5, 16.5
 //             216,000: 21.5 / 24.1, 22.1 238,328: 23.4 / 25.6, 23.8 262,144: 27.0 / 28.8, 27.1
+// Reverse sweep, 128 threads a block, early / after:
+//   flow         7200: 31.0 / 33.4      13,824: 72.1 / 33.5     46,656: 76.7 / 66.2
+//              64,000: 73.0 / 74.4
+//   conduction 18,954: 12.0 / 12.9      24,389: 18.2 / 15.6    129,792: 43.2 / 33.5
+//             216,000: 49.3 / 51.5
 template <int P>
-inline bool start_early(const Args& a) {
+inline bool start_early(const Args& a, bool reverse = false) {
     if (P != LBPC_FP64) return true;
-    return a.flow ? a.N <= 43 * SM_COUNT || a.N >= 320 * SM_COUNT
-                  : a.N <= 128 * SM_COUNT || a.N >= 832 * SM_COUNT;
+    return a.flow ? a.N <= 43 * SM_COUNT || a.N >= (reverse ? 384 : 320) * SM_COUNT
+                  : a.N <= 128 * SM_COUNT || a.N >= (reverse ? 1408 : 832) * SM_COUNT;
 }
 template <int P>
 inline ItemGrid step_grid(const Args& a) {
@@ -2999,7 +3004,7 @@ struct Impl {
                 return;
             }
         }
-        launch_after(a.flow ? k_adj_reverse<P, true> : k_adj_reverse<P, false>, node_grid(a), start_early<P>(a), s, a,
+        launch_after(a.flow ? k_adj_reverse<P, true> : k_adj_reverse<P, false>, node_grid(a), start_early<P>(a, true), s, a,
                      (const C*)lin, (C*)lout, (const C*)tape_e, (const C*)tape_m, wface, gtw,
                      Lpart);
     }
