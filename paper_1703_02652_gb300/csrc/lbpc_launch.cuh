@@ -28,19 +28,23 @@ LBPC_HD void opaque(T& v) {
 }
 
 #if defined(__CUDACC__)
-// In the kernels that follow one another on a stream, before any access to their data: lets
-// the next grid of the stream become resident while this one drains, then waits until the
-// previous grid has completed and its stores are visible.  The pointers given go through the
-// barrier.  A __restrict__ pointer has to: the compiler may take it that nothing else, the
-// barrier included, touches its data, and move a load above.  Others are held by the memory
-// clobber; those that the pair kernels pass all the same are a measurement (addresses are then
-// formed after the barrier: up to 8% of a 16-bit step either way).
+// In the kernels that follow one another on a stream, before any access to their data: waits
+// until the previous grid has completed and its stores are visible, then lets the next grid of
+// the stream become resident while this one works.  In this order: a grid that let the next one
+// in before it waits would have a whole call's grids queue up on the SMs, each of them putting its
+// blocks where a waiting one left room (128 x 1 x 128 FP64 conduction, us a step: 4.8 in a call
+// of 50 steps, 12.2 in one of 1000; in this order 3.7 and 3.9, without overlap 6.2).
+// The pointers given go through the barrier.  A __restrict__ pointer has to: the compiler may
+// take it that nothing else, the barrier included, touches its data, and move a load above.
+// Others are held by the memory clobber; those that the pair kernels pass all the same are a
+// measurement (addresses are then formed after the barrier: up to 8% of a 16-bit step either
+// way).
 // Why: between two dependent launches the GPU waits in steps of about 2 us; 64^3 FP32 took
-// 10.3 us a step without the overlap and 8.0 us with it (6.2 -> 3.1 us at 64 x 1 x 64).
+// 10.3 us a step without the overlap and 8.1 us with it (4.1 -> 2.3 us for 32^3 conduction).
 template <class... Ptr>
 __device__ __forceinline__ void after_previous_grid(Ptr&... p) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     (opaque(p), ...);
 }
 
