@@ -2768,37 +2768,41 @@ k_adj_reverse_x2(const __grid_constant__ Args a, const CT<P>* __restrict__ lin,
 // ---------------------------------------------------------------------------------
 // Host launchers.
 // ---------------------------------------------------------------------------------
-// FP64 lattices.  Grids of some warps per SM start after the one before instead: early blocks go
-// where that one left room, several to an SM beside idle ones, and share its FP64 pipe.  Up to
-// about one warp per scheduler (conduction) or per SM (flow) there is nothing to share, and large
-// grids fill every SM whenever they start.  Blocks of one warp spread best until there are many
-// per SM.  us a step, early / after with 32 threads a block, and the better of the two with 128
-// (cubes and n x 1 x n planes agree within 10%):
-//   flow         4624: 8.9 / 10.4, 8.8     6498: 9.0 / 10.3, 8.8      7200: 10.6 / 10.3, 8.7
-//                8000: 9.2 / 10.3, 10.3    9000: 13.0 / 10.3, 10.3   32,768: 17.5 / 14.4, 14.4
-//              46,656: 18.1 / 17.8, 18.1  49,152: 18.0 / 18.5, 18.0  57,798: 18.5 / 20.6, 18.4
-//             175,616: 50.9 / 53.4, 52.9 262,144: 73.2 / 75.8, 72.8
-//   conduction 13,824: 4.4 / 6.2, 5.4     19,200: 4.8 / 6.2, 4.7     20,480: 7.9 / 6.2, 6.1
-//              64,000: 12.9 / 10.3, 10.3 122,500: 15.5 / 14.6, 16.5 128,000: 16.2 / 16.5, 16.5
-//             216,000: 21.5 / 24.1, 22.1 238,328: 23.4 / 25.6, 23.8 262,144: 27.0 / 28.8, 27.1
+// FP64 lattices.  An early grid puts its blocks beside those of the grid at work, so it spreads like
+// that one as long as both fit: up to half of the blocks that an SM holds (16 of 32 blocks of one
+// warp in conduction, 6 of 12 warps with flow; reverse sweep 16 and 8 warps).  Above, its last
+// blocks pile up on the SMs that finish first and share their FP64 pipe beside idle ones, until a
+// grid fills the device several times and it no longer matters.  In between a grid starts after
+// the one before.  Blocks of one warp spread best until there are many per SM.
+// us a step in calls of 600 steps, early / after with 32 threads a block, and the better of the
+// two with 128 (cubes; n x 1 x n planes agree within 10%):
+//   conduction 24^3: 3.7 / 6.2, 3.8     40^3: 7.7 / 10.3, 8.3   72,324: 8.3 / 10.3, 8.3
+//              43^3: 15.2 / 12.3, 10.0  46^3: 15.2 / 14.3, 14.3  122,500: 15.3 / 14.6, 16.4
+//           127,449: 15.3 / 16.4, 16.4  62^3: 23.3 / 25.8, 23.7  64^3: 25.1 / 26.7, 25.3
+//   flow       20^3: 8.6 / 10.3, 8.6    26^3: 9.0 / 10.3, 8.8   30^3: 11.3 / 13.8, 12.8
+//              31^3: 18.0 / 14.3, 14.4  34^3: 18.2 / 16.4, 17.8  36^3: 18.0 / 18.3, 17.8
+//              40^3: 23.2 / 25.1, 28.1  62^3: 68.1 / 70.0, 70.1  64^3: 73.5 / 75.8, 73.1
 // Reverse sweep, 128 threads a block, early / after:
-//   flow         7200: 31.0 / 33.4      13,824: 72.1 / 33.5     46,656: 76.7 / 66.2
-//              64,000: 73.0 / 74.4
-//   conduction 18,954: 12.0 / 12.9      24,389: 18.2 / 15.6    129,792: 43.2 / 33.5
-//             216,000: 49.3 / 51.5
-template <int P>
-inline bool start_early(const Args& a, bool reverse = false) {
-    if (P != LBPC_FP64) return true;
-    return a.flow ? a.N <= 43 * SM_COUNT || a.N >= (reverse ? 384 : 320) * SM_COUNT
-                  : a.N <= 128 * SM_COUNT || a.N >= (reverse ? 1408 : 832) * SM_COUNT;
-}
+//   conduction 32^3: 9.9 / 12.5         72,324: 20.2 / 22.7     44^3: 30.9 / 26.9
+//              53^3: 43.0 / 37.1        60^3: 48.8 / 51.3
+//   flow       29^3: 45.6 / 47.5        192 x 1 x 192: 31.1 / 33.1  36^3: 76.6 / 65.9
+//              38^3: 76.2 / 59.9        256 x 1 x 256: 59.0 / 61.8
 template <int P>
 inline ItemGrid step_grid(const Args& a) {
-    const bool one_warp = P == LBPC_FP64 && a.N < 12 * STEP_THREADS * SM_COUNT;
+    const bool one_warp = P == LBPC_FP64 && a.N < 1600 * SM_COUNT;
     return item_grid(a.nx, a.ny, a.nz, one_warp ? 32 : STEP_THREADS);
 }
 inline ItemGrid node_grid(const Args& a) { return item_grid(a.nx, a.ny, a.nz); }
 inline ItemGrid pair_grid(const Args& a) { return item_grid(a.nx / 2, a.ny, a.nz); }
+template <int P>
+inline bool start_early(const Args& a, const ItemGrid& g, bool reverse = false) {
+    if (P != LBPC_FP64) return true;
+    const long long blocks = (long long)g.grid.x * g.grid.y * g.grid.z;
+    const long long warps = blocks * (g.block.x * g.block.y / 32);
+    if (a.flow)
+        return warps <= (reverse ? 8 : 6) * SM_COUNT || a.N >= (reverse ? 416 : 300) * SM_COUNT;
+    return warps <= 16 * SM_COUNT || a.N >= (reverse ? 1408 : 832) * SM_COUNT;
+}
 
 template <int P>
 struct Impl {
@@ -2822,7 +2826,7 @@ struct Impl {
                 return;
             }
         }
-        launch_after(k_step<P, KIND, FLOW, TAPE>, step_grid<P>(a), start_early<P>(a), s, a, (const T*)fs, (T*)fd,
+        launch_after(k_step<P, KIND, FLOW, TAPE>, step_grid<P>(a), start_early<P>(a, step_grid<P>(a)), s, a, (const T*)fs, (T*)fd,
                      (const TGp*)gs, (TGp*)gd, hp, (C*)tape_e, (C*)tape_m);
     }
     static void step(const Args& a, StepKind kind, const void* fs, void* fd, const void* gs,
@@ -3004,7 +3008,7 @@ struct Impl {
                 return;
             }
         }
-        launch_after(a.flow ? k_adj_reverse<P, true> : k_adj_reverse<P, false>, node_grid(a), start_early<P>(a, true), s, a,
+        launch_after(a.flow ? k_adj_reverse<P, true> : k_adj_reverse<P, false>, node_grid(a), start_early<P>(a, node_grid(a), true), s, a,
                      (const C*)lin, (C*)lout, (const C*)tape_e, (const C*)tape_m, wface, gtw,
                      Lpart);
     }
