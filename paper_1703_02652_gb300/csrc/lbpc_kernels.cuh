@@ -2384,7 +2384,7 @@ k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* hp) {
 // ---------------------------------------------------------------------------------
 // Small lattices: a block of steps in one launch.
 //
-// A lattice of a few thousand nodes is bound by latency: one launch per step costs 3-4 us
+// A lattice of a few thousand nodes is bound by latency: one launch per step costs 2-4 us
 // even with its start overlapped, most of it the way to the L2 and back.  One cluster of
 // CL_CTAS CTAs keeps the whole lattice on chip instead: thread l of CTA c owns node
 // c * per + l for all n steps, its rest channel stays in a register, and the populations go
@@ -2393,13 +2393,14 @@ k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* hp) {
 // shared memory.  One hardware cluster barrier per step orders the exchange: step i writes
 // buffer i % 2, which the step before it read and every CTA has since left.  The first
 // gather and the last scatter are the per-node path's, in the layout that the handle holds.
-// Measured, us a step before and after: 64 x 1 x 64 FP32 3.4 and 1.1, 64 x 4 x 4 FP64
-// conduction 3.7 and 2.3, 57 x 1 x 92 FP32 3.4 and 1.4.
+// us a step, pull, single steps and in blocks of 400: FP32 16^3 3.2 and 1.4, 8192 nodes 3.1 and
+// 2.3; conduction FP32 16^3 2.3 and 1.0, 8192 nodes 2.3 and 1.3; FP16 2.1 and 0.8, 2.1 and 1.0; FP64
+// 512 nodes 3.9 and 2.2, 3072 nodes 3.7 and 3.1, 4096 nodes 3.6 and 3.9.
 // ---------------------------------------------------------------------------------
 constexpr int CL_CTAS = 16;      // one GPC; more than 8 needs the non-portable attribute
 // nodes of a CTA at most: the lattice sizes up to which the cluster beats the step-by-step
-// path (3-4 us a step, spread over all SMs).  FP64 collisions are bound by the FP64 pipe of
-// the 16 SMs.
+// path (figures above; in FP64 they meet at 3700 nodes).  FP64 collisions are bound by the
+// FP64 pipe of the 16 SMs.
 template <int P, bool FLOW>
 constexpr int CL_THREADS = P == LBPC_FP64 && !FLOW ? 256 : 512;
 
