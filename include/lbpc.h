@@ -188,7 +188,7 @@ lbpc_status lbpc_set_wall_temperature(lbpc_handle *h, int face, const double *T_
  * 50 (flow, collision Eq. 49 with Eq. 51-54), coupled through Eq. 2, Eq. 55 and Eq. 56,
  * with the walls of Sec. 3.1-3.3.  Small lattices may take four or more steps in one launch,
  * with the bits of the same steps one by one: up to 8192 nodes in FP32 (without the drag
- * closure) and, without flow, in 16-bit storage, up to 4096 nodes in FP64 without flow, on a
+ * closure) and, without flow, in 16-bit storage, up to 3584 nodes in FP64 without flow, on a
  * device that holds a cluster of 16 blocks; a launch ends at a diagnostics point and after
  * 2048 steps.  Divergence checks: with report_every > 0 the call is
  * asynchronous unless it passes a diagnostics point; then it waits for the stream and

@@ -2399,10 +2399,10 @@ k_step_aa_x2(const __grid_constant__ Args a, TF<P>* F, TG<P>* G, double* hp) {
 // ---------------------------------------------------------------------------------
 constexpr int CL_CTAS = 16;      // one GPC; more than 8 needs the non-portable attribute
 // nodes of a CTA at most: the lattice sizes up to which the cluster beats the step-by-step
-// path (figures above; in FP64 they meet at 3700 nodes).  FP64 collisions are bound by the
+// path (figures above; in FP64 the two meet near 3600 nodes).  FP64 collisions are bound by the
 // FP64 pipe of the 16 SMs.
 template <int P, bool FLOW>
-constexpr int CL_THREADS = P == LBPC_FP64 && !FLOW ? 256 : 512;
+constexpr int CL_THREADS = P == LBPC_FP64 && !FLOW ? 224 : 512;
 
 __device__ __forceinline__ unsigned shared_at(const void* p, unsigned cta) {
     unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
